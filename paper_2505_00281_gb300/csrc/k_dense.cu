@@ -170,7 +170,7 @@ extern "C" rr_status rr_cast_operator(int64_t m, int64_t n, const double* A, int
   switch (dtype) {
     case RR_F32: k_cast_operator<float><<<g, b, 0, s>>>(m, n, A, lda, (float*)out_col, (float*)out_row); break;
     case RR_BF16:
-      return op_prepare(s, A, m, n, lda, (__nv_bfloat16*)out_col, (__nv_bfloat16*)out_row, nullptr, nullptr, 0,
+      return op_prepare(s, A, m, n, lda, (__nv_bfloat16*)out_col, (__nv_bfloat16*)out_row, nullptr, nullptr,
                         nullptr, nullptr, false, false);
     case RR_F64: k_cast_operator<double><<<g, b, 0, s>>>(m, n, A, lda, (double*)out_col, (double*)out_row); break;
     default: return RR_ERR_ARG;
@@ -440,13 +440,11 @@ static int64_t gram_chunks(int64_t n, int64_t p, int64_t q) {
 }  // namespace rr
 
 // Workspace: the SIMT path's split-K partials, or the tensor-core path's
-// slices and partials when the shape qualifies (for q > 128 the calls with
-// q' <= 128 columns qualify)
+// exponents and partial tiles when the shape qualifies
 extern "C" size_t rr_gram_workspace_size(int64_t n, int64_t p, int64_t q) {
   size_t b = align_up((size_t)gram_chunks(n, p, q) * p * q * sizeof(double)) + 256;
-  const int64_t qe = q < 128 ? q : 128;
-  if (emu_gram_supported(n, p, qe)) {
-    const size_t e = emu_gram_bytes(n, p, qe);
+  if (emu_gram_supported(n, p, q)) {
+    const size_t e = emu_gram_bytes(n, p, q);
     if (e > b) b = e;
   }
   return b;
@@ -647,20 +645,9 @@ extern "C" rr_status rr_gram(int64_t n, int64_t p, int64_t q, int32_t xtype, con
     return RR_OK;
   }
   // FP64-accurate products on the tensor cores when the shape qualifies and
-  // the workspace holds the slices
+  // the workspace holds the partial tiles
   if (emu_gram_supported(n, p, q) && ws && ws_bytes >= emu_gram_bytes(n, p, q))
     return emu_gram(s, n, p, q, xtype, X, ldx, ytype, Y, ldy, G, ldg, accumulate, ws, ws_bytes);
-  // wider Y: the same products on column chunks of at most 128
-  constexpr int64_t kQc = 128;
-  if (q > kQc && emu_gram_supported(n, p, kQc) && ws && ws_bytes >= emu_gram_bytes(n, p, kQc)) {
-    const size_t ys = dtype_size(ytype);
-    for (int64_t j0 = 0; j0 < q; j0 += kQc) {
-      const int64_t qc = std::min<int64_t>(kQc, q - j0);
-      RR_TRY(emu_gram(s, n, p, qc, xtype, X, ldx, ytype, (const char*)Y + (size_t)j0 * ldy * ys, ldy, G + j0 * ldg,
-                      ldg, accumulate, ws, ws_bytes));
-    }
-    return RR_OK;
-  }
   int64_t chunks = gram_chunks(n, p, q);
   if (ws_bytes < (size_t)chunks * p * q * sizeof(double) || !ws) return RR_ERR_WORKSPACE;
   int64_t rpc = (n + chunks - 1) / chunks;

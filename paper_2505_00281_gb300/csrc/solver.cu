@@ -230,7 +230,7 @@ static rr_status apply_f64(const Op& op, int64_t b, const double* X, int64_t ldx
   if (op.kind == RR_KERNEL)
     return kernel_apply(s, op.kop, 0, b, RR_F64, X, ldx, RR_F64, out, ldo, nullptr, 0, nullptr);
   if (op.kind == RR_DENSE) {
-    if (op.has_emu && b <= 256) return emu_gemm(s, op.emu, 0, b, X, ldx, out, ldo, op.emu_blk);
+    if (op.has_emu && b <= 256) return emu_gemm(s, op.emu, 0, b, X, ldx, out, ldo, kEmuSlices, op.emu_blk);
     return rr_gemm_f64(0, op.m, b, op.n, op.A, op.lda, X, ldx, out, ldo, 0, s);
   }
   return rr_csr_spmm(op.n, b, op.rp, op.ci, op.va, RR_F64, X, ldx, RR_F64, out, ldo, s);
@@ -240,7 +240,8 @@ static rr_status apply_f64_T(const Op& op, int64_t b, const double* X, int64_t l
   if (op.kind == RR_KERNEL)
     return kernel_apply(s, op.kop, 1, b, RR_F64, X, ldx, RR_F64, out, ldo, nullptr, 0, nullptr);
   if (op.kind != RR_DENSE) return RR_ERR_ARG;
-  if (op.has_emu && op.emu.cols && b <= 256) return emu_gemm(s, op.emu, 1, b, X, ldx, out, ldo, op.emu_blk);
+  if (op.has_emu && op.emu.cexp && b <= 256)
+    return emu_gemm(s, op.emu, 1, b, X, ldx, out, ldo, kEmuSlices, op.emu_blk);
   return rr_gemm_f64(1, op.n, b, op.m, op.A, op.lda, X, ldx, out, ldo, 0, s);
 }
 
@@ -561,7 +562,7 @@ static void carve_op(Arena& ar, Op& op, bool symmetric, bool refine, int64_t b) 
   }
   if (refine && op.m % 8 == 0 && op.n % 8 == 0 && b <= 256) {
     op.has_emu = true;
-    op.emu_mem = ar.take_bytes(emu_operator_bytes(op.m, op.n, kEmuSlices, true, !symmetric));
+    op.emu_mem = ar.take_bytes(emu_operator_bytes(op.m, op.n, true, !symmetric));
     op.emu_blk = ar.take_bytes(emu_block_bytes(op.m > op.n ? op.m : op.n, b, kEmuSlices));
   }
 }
@@ -574,19 +575,19 @@ static rr_status prepare_f8(const Op& op, int64_t b, cudaStream_t s) {
 
 static rr_status prepare_op(const Op& op_in, Op& op, bool symmetric, cudaStream_t s) {
   (void)op_in;
-  if (op.kind == RR_DENSE && op.dt == RR_BF16 && op.lo_col && (!op.has_emu || kEmuSlices == 8)) {
+  if (op.kind == RR_DENSE && op.dt == RR_BF16 && op.lo_col) {
     // every copy and slice of the operator from two passes over A
     return op_prepare(s, op.A, op.m, op.n, op.lda, (__nv_bfloat16*)op.lo_col,
                       symmetric ? nullptr : (__nv_bfloat16*)op.lo_row,
                       op.split ? (__nv_bfloat16*)op.lo2_col : nullptr,
-                      op.split && !symmetric ? (__nv_bfloat16*)op.lo2_row : nullptr, kEmuSlices,
+                      op.split && !symmetric ? (__nv_bfloat16*)op.lo2_row : nullptr,
                       op.has_emu ? &op.emu : nullptr, op.emu_mem, true, !symmetric);
   }
   if (op.lo_col)
     RR_TRY(rr_cast_operator(op.m, op.n, op.A, op.lda, op.dt, op.lo_col, symmetric ? nullptr : op.lo_row, s));
   if (op.split) RR_TRY(cast_operator_lo(op.m, op.n, op.A, op.lda, op.lo2_col, op.lo2_row, s));
   if (op.has_emu)
-    RR_TRY(emu_prepare(s, op.A, op.m, op.n, op.lda, kEmuSlices, op.emu, op.emu_mem, true, !symmetric));
+    RR_TRY(emu_prepare(s, op.A, op.m, op.n, op.lda, op.emu, op.emu_mem, true, !symmetric));
   return RR_OK;
 }
 

@@ -57,9 +57,9 @@ rr_status fill_f32(cudaStream_t s, int64_t n, float v, float* d);
 // Upper bound on the K splits of the plain / split tensor-core products
 // (0: none) while an instance is alive on this thread; the batched solver
 // sets it around its graph capture.
-// Kernel-level timing of the tensor-core product kernel (k_gemm_bf16_tc in
-// every role: filter products, split corrections, FP64 emulation passes,
-// E4M3 products): while a TcProf is attached to the calling thread, each
+// Kernel-level timing of the tensor-core product kernels (k_gemm_bf16_tc:
+// filter products, split corrections, E4M3 products; k_emu_mm: FP64-accurate
+// products): while a TcProf is attached to the calling thread, each
 // launch is bracketed by CUDA events on its stream and its algorithmic bytes
 // (each operand read once, the output written once) are added up.
 struct TcProf {
@@ -71,6 +71,13 @@ struct TcProf {
   int launches = 0;
 };
 void tc_prof_attach(TcProf* p);  // nullptr detaches
+// event pair around one tensor-core launch (nothing while no TcProf is attached)
+struct TcProfScope {
+  TcProf* p;
+  cudaStream_t s;
+  TcProfScope(cudaStream_t s, double bytes, double flops, int role);
+  ~TcProfScope();
+};
 // the small pencils' side stream for the caller stream s (created here if new;
 // call before capturing work on s)
 rr_status pencil_side_prepare(cudaStream_t s);
@@ -113,58 +120,37 @@ rr_status sub_block_f32(cudaStream_t s, int64_t n, int64_t b, const float* P, in
 rr_status tc_take_error(cudaStream_t s);
 rr_status tc_prepare_attributes();
 
-// Tensor-core launch of an FP64-emulation product (k_gemm_tc.cu): the sum
-// over slice pairs (pair[z] = p0 | q0 << 8 | nq << 16, 0-based) of the A
-// slice p0 times B slices q0 (and q0 + 1 when nq = 2), element (row, col)
-// scaled by 2^(rexp[row] + cexp[col] - 6 (p0 + 1) - 6 (q0 + nq)); added into
-// C64 (ld ldc64) or written as one M x nb partial (ld M) per (pair, K split).
-struct TcEmu {
-  double* C64;
-  int64_t ldc64;
-  double* part;
-  const int* rexp;
-  const int* cexp;
-  int nb;
-  int a_slices, b_slices;          // slices stacked in the A / B operands
-  int a_slice_rows, b_slice_rows;  // rows of one slice in the tensor-map outer dimension
-  int npairs;                      // <= 48
-  const uint32_t* pair;            // host array
-  int max_kchunk;                  // K elements per exact FP32 accumulation
-  // > 0: a lift's anti-diagonal products in one launch (pair z codes diagonal
-  // d = p0 + 2 of lift_s): A's K range [0, (p0 + 1) lift_k0), B's
-  // [(lift_s - 1 - p0) lift_k0, lift_s lift_k0); K = lift_s lift_k0
-  int lift_k0, lift_s;
-};
-rr_status gemm_bf16_tc_emu(int64_t M, int64_t N, int64_t K, const __nv_bfloat16* A, int64_t lda,
-                           const __nv_bfloat16* B, int64_t ldb, const TcEmu& e, cudaStream_t s);
-int tc_emu_partial_splits(int64_t M, int64_t K, int npairs, int max_kchunk);
 rr_status gemm_bf16_tc_split(int64_t M, int64_t N, int64_t K, const __nv_bfloat16* A_hi,
                              const __nv_bfloat16* A_lo, int64_t lda, const __nv_bfloat16* B_hi,
                              const __nv_bfloat16* B_lo, int64_t ldb, float* C, int64_t ldc,
                              const double* R, int64_t ldr, const double* coef, cudaStream_t s);
 
-// FP64-accurate products on the tensor cores (k_f64emu.cu)
+// FP64-accurate products on the tensor cores (k_emu_mm.cu): a dense FP64
+// operator (not copied: it must outlive the struct) with the exponents of its
+// largest entry per row (for A X) and per column (for A^T Y)
 struct EmuOperator {
   int64_t m, n;
-  int S;
-  __nv_bfloat16* rows;  // S row-scaled slices, row-major (for A X)
+  const double* A;
+  int64_t lda;
   int* rexp;
-  __nv_bfloat16* cols;  // S column-scaled slices, column-major (for A^T Y)
   int* cexp;
 };
-size_t emu_operator_bytes(int64_t m, int64_t n, int S, bool rows, bool cols);
-size_t emu_block_bytes(int64_t K, int64_t N, int S);
-rr_status emu_prepare(cudaStream_t s, const double* A, int64_t m, int64_t n, int64_t lda, int S,
-                      EmuOperator& op, void* mem, bool rows, bool cols);
+size_t emu_operator_bytes(int64_t m, int64_t n, bool rows, bool cols);
+size_t emu_block_bytes(int64_t K, int64_t N, int slices);
+rr_status emu_prepare(cudaStream_t s, const double* A, int64_t m, int64_t n, int64_t lda, EmuOperator& op, void* mem,
+                      bool rows, bool cols);
+rr_status emu_prepare_attributes();
+rr_status emu_error_fetch(cudaStream_t s, int* host);
+rr_status emu_error_clear(cudaStream_t s);
 size_t lift_emu_bytes(int64_t n, int64_t b, int64_t K);
 rr_status lift_emu(cudaStream_t s, int64_t n, int64_t b, int32_t t1, const void* S1, int64_t ld1, int64_t p1,
                    int32_t t2, const void* S2, int64_t ld2, int64_t p2, const double* Y, int64_t ldy, double* X,
                    int64_t ldx, void* mem, size_t mem_bytes, bool* done);
 rr_status op_prepare(cudaStream_t s, const double* A, int64_t m, int64_t n, int64_t lda,
                      __nv_bfloat16* hi_col, __nv_bfloat16* hi_row, __nv_bfloat16* lo_col, __nv_bfloat16* lo_row,
-                     int S, EmuOperator* emu, void* emu_mem, bool rows, bool cols);
+                     EmuOperator* emu, void* emu_mem, bool rows, bool cols);
 rr_status emu_gemm(cudaStream_t s, const EmuOperator& op, int trans, int64_t N, const double* X,
-                   int64_t ldx, double* C, int64_t ldc, void* mem);
+                   int64_t ldx, double* C, int64_t ldc, int slices, void* mem);
 rr_status vec_scale(cudaStream_t s, int64_t n, double alpha, const double* a, double* d);
 bool emu_gram_supported(int64_t n, int64_t p, int64_t q);
 size_t emu_gram_bytes(int64_t n, int64_t p, int64_t q);
