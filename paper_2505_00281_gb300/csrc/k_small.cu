@@ -762,18 +762,26 @@ __global__ void k_whiten_corr(int b, double* __restrict__ E, const double* __res
 // blocks (sub-round t pairs column i of block a with column (i + t) mod w of
 // block b), c - 1 sub-rounds per sweep in all.
 //
-// In a sub-round warp i forms the inner product of its pair (in the cross
-// rounds column i of block a stays in warp i's registers for the whole
-// round), computes the rotation, carries the squared column norms through it
-// (|x'|^2 = |x|^2 - t g, |y'|^2 = |y|^2 + t g; the norms are computed when
-// the block is loaded) and applies it to the pair and to the round's 2w x 2w
-// accumulated rotation Q, which is applied to the V block once at the end of
-// the round (V_blk <- V_blk Q); the pairs of a sub-round are disjoint, so one
-// __syncthreads separates sub-rounds.  A pair whose
-// inner product is exactly zero, or below tol relative to the column norms
-// (floored, so rounding-level columns count as converged against
-// everything), is not rotated; zero columns (dropped directions, padding)
-// stay decoupled.  Converged when a sweep rotates nothing.
+// A round works on the 2w x 2w Gram matrix of its columns, formed once per
+// round: a sub-round's disjoint pairs take their rotations from it, it is
+// updated on both sides by 2 x 2 blocks (into a second copy), and the rotations
+// collect in Q, which then multiplies the M and V blocks.  The chain of a
+// sub-round (c - 1 of them per sweep, one after the other) is what bounds the
+// kernel: one warp works out the next sub-round's rotations, from the Gram
+// entries as they were before this one, while others apply this one's, so a
+// sub-round is one barrier apart from the next.  A round of 2 x 16 columns of
+// 256 rows takes some 15 thousand clocks (Gram matrix 2.7, 16 sub-rounds of 370
+// clocks, products and exchange 5.1, cluster barrier 2.6) where full-length
+// inner products and column updates in every sub-round took 32 thousand:
+// rr_pencil_svd at 256 x 256 from 5.25 to 4.26 ms, at 320 x 320 (a barrier over
+// the grid instead of the cluster's) from 9.1 to 8.1 ms.
+// The rounding of the Gram entries is relative to the two columns' norms, far
+// below the 1e-4 the Jacobi stops at, and the next round starts from fresh
+// ones.  A pair whose inner product is exactly zero, or below tol relative to
+// the column norms (floored, so rounding-level columns count as converged
+// against everything), is not rotated; zero columns (dropped directions,
+// padding) stay decoupled.  A round none of whose pairs would rotate skips its
+// sub-rounds; converged when that holds for a whole sweep.
 constexpr int kBJThreads = 512;
 constexpr int kBJMaxChunks = 3;  // float4 row chunks per lane: r, cpad <= 384
 
@@ -798,115 +806,364 @@ __device__ __forceinline__ void bj_pair(int round, int pi, int sr, int w, int& p
   }
 }
 
-// One round's pair work on the 2w columns in shared memory (Ms [2w][rp],
-// tracked squared norms nrm, Q accumulated in Qs [2w][ldq]); every thread of
-// the block calls it, and it ends with the columns back in Ms.
-template <int NCH>
-__device__ __forceinline__ void bj_round(int round, int w, int rp, float* __restrict__ Ms, float* __restrict__ Qs,
-                                         int ldq, float* __restrict__ nrm, float nfloor, float tol2,
-                                         int* s_rot) {
+// a b + c on two values
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
+  unsigned long long x, y, z;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(x) : "f"(a.x), "f"(a.y));
+  asm("mov.b64 %0, {%1, %2};" : "=l"(y) : "f"(b.x), "f"(b.y));
+  asm("mov.b64 %0, {%1, %2};" : "=l"(z) : "f"(c.x), "f"(c.y));
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(z) : "l"(x), "l"(y), "l"(z));
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(c.x), "=f"(c.y) : "l"(z));
+  return c;
+}
+
+// rotate unless |g| <= tol |x| |y| (squared form; the block is scaled so that
+// squared norms stay far from the FP32 range limits)
+__device__ __forceinline__ bool bj_rotates(float al, float be, float ga, float nfloor, float tol2) {
+  return ga != 0.f && ga * ga > tol2 * fmaxf(al, nfloor) * fmaxf(be, nfloor);
+}
+
+__device__ __forceinline__ float bj_rsqrt(float x) {
+  float y;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+
+// Rotation of a pair with squared norms al, be and inner product ga:
+// x' = cs x - sn y, y' = sn x + cs y orthogonal, |angle| <= pi/4
+// (cos 2a = |be - al| / h, sin 2a = 2 ga / h, h^2 = (be - al)^2 + 4 ga^2;
+// the floor keeps h^2 of a rotated pair far above the smallest FP32 value);
+// the identity when the pair is not rotated.  tn = sn / cs.
+__device__ __forceinline__ void bj_rotation(float al, float be, float ga, float nfloor, float tol2, float& cs,
+                                            float& sn, float& tn) {
+  const bool rot = bj_rotates(al, be, ga, nfloor, tol2);
+  const float d = be - al, g2 = 2.f * ga;
+  const float ih = bj_rsqrt(fmaf(d, d, g2 * g2));
+  const float c2 = fmaf(0.5f * fabsf(d), ih, 0.5f);  // cos^2
+  const float rc = bj_rsqrt(c2);
+  const float sg = (d < 0.f ? -ga : ga) * ih;
+  float c = c2 * rc, t = sg * rc * rc;
+  float sv = sg * rc;
+  const float f = fmaf(-0.5f, fmaf(c, c, sv * sv), 1.5f);  // one Newton step: cs^2 + sn^2 = 1
+  cs = rot ? c * f : 1.f;
+  sn = rot ? sv * f : 0.f;
+  tn = rot ? t : 0.f;
+}
+
+// Row stride of Q and of the Gram matrix in shared memory: 16 modulo 32 banks,
+// so that a warp's two rows of 16 columns take all banks once.
+constexpr int kBJLd = 48;
+
+// Inner products of columns 4 a .. 4 a + 3 and 4 b .. 4 b + 3 of Ms [.][4 rch]
+// (columns from `last` on repeat it), over the row chunks l, l + kL, ...: each
+// lane's share, then summed over the kL = 8 or 32 lanes of a group, halving the
+// values a lane keeps at each step: lane l of the group ends with entries
+// l * 16 / kL .. of the tile (kL = 32: lanes l and l + 16 the same).
+template <int kL>
+__device__ __forceinline__ void bj_gram_tile(const float* __restrict__ Ms, int rch, int ca, int cb, int lasta,
+                                             int lastb, bool on, float (&v)[16]) {
+  const int lane = threadIdx.x & 31;
+  float2 acc[4][4];  // rows 4 ch, 4 ch + 2 | rows 4 ch + 1, 4 ch + 3
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) acc[i][j] = make_float2(0.f, 0.f);
+  if (on) {
+    const float4* xp[4];
+    const float4* yp[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      xp[i] = reinterpret_cast<const float4*>(Ms) + (size_t)min(ca + i, lasta) * rch;
+      yp[i] = reinterpret_cast<const float4*>(Ms) + (size_t)min(cb + i, lastb) * rch;
+    }
+#pragma unroll 2
+    for (int ch = lane & (kL - 1); ch < rch; ch += kL) {
+      float4 x[4], y[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        x[i] = xp[i][ch];
+        y[i] = yp[i][ch];
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          acc[i][j] = fma2(make_float2(x[i].x, x[i].y), make_float2(y[j].x, y[j].y), acc[i][j]);
+          acc[i][j] = fma2(make_float2(x[i].z, x[i].w), make_float2(y[j].z, y[j].w), acc[i][j]);
+        }
+    }
+  }
+#pragma unroll
+  for (int e = 0; e < 16; ++e) v[e] = acc[e >> 2][e & 3].x + acc[e >> 2][e & 3].y;
+  constexpr int kSteps = kL == 32 ? 4 : 3;
+#pragma unroll
+  for (int st = 0; st < kSteps; ++st) {
+    const int h = 8 >> st, m = (1 << (kSteps - 1)) >> st;
+    const bool hi = (lane & m) != 0;
+#pragma unroll
+    for (int e = 0; e < 8; ++e)
+      if (e < h) {
+        const float keep = hi ? v[e + h] : v[e], send = hi ? v[e] : v[e + h];
+        v[e] = keep + __shfl_xor_sync(0xffffffffu, send, m);
+      }
+  }
+  if (kL == 32) v[0] += __shfl_xor_sync(0xffffffffu, v[0], 16);
+}
+
+// barrier over the warps that work in the sub-rounds (13 of the 16)
+constexpr int kBJSubThreads = 416;
+__device__ __forceinline__ void bj_sub_barrier() {
+  asm volatile("bar.sync 1, %0;" ::"n"(kBJSubThreads) : "memory");
+}
+
+constexpr int kBJGs = 32 * kBJLd;  // floats from one copy of the Gram matrix to the other
+
+// The sub-rounds of a round on the Gram matrix in Gs (the second copy kBJGs
+// behind it; sub-round sr reads copy sr & 1 and writes the other), Q <- Q J.
+// kR0: round 0's pairs (all among the 2w columns) or the cross pairs.
+//   warp 0          the next sub-round's rotations (lane = pair)
+//   warps 4 .. 11   the Gram matrix's 2 x 2 blocks of pairs (a, b)
+//   warps 12 .. 15  Q, rows i0, i0 + nr, ... in pair b's columns
+// each in a loop of its own: the instructions issued per sub-round set its pace
+// next to the chain of warp 0.  s_rt [2][16]: cs, sn, sn / cs and the inner
+// product of a sub-round's pairs, by parity.  al, be, ga, cs, sn, tn: the
+// lane's pair in warp 0.
+template <bool kR0>
+__device__ __forceinline__ void bj_subs(int w, float* __restrict__ Qs, float* __restrict__ Gs, float4 (*s_rt)[16],
+                                        float nfloor, float tol2, float al, float be, float ga, float cs, float sn,
+                                        float tn) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, w2 = 2 * w;
+  const int nsub = kR0 ? w2 - 1 : w;
+  if (warp == 0) {
+    const int i = lane < w ? lane : 0;
+    const unsigned all = 0xffffffffu;
+    const int Yc = add_mod(i, 1, w);
+    int qx = w + i, qy = w + Yc;
+    for (int sr = 0; sr + 1 < nsub; ++sr) {
+      // the next sub-round's pair (x, y) of this lane: x is in this one's
+      // pair X, y in pair Y (X != Y), as its first or second column
+      const float* G = Gs + ((sr & 1) ? kBJGs : 0);
+      const float an = fmaf(-tn, ga, al), bn = fmaf(tn, ga, be);  // the lane's pair after its rotation
+      if (kR0) {
+        int X = i == 0 ? 0 : min(i + 1, w - 1), Y = i == 0 ? 1 : i - 1;
+        int x, y, px, py;
+        bj_pair(0, i, sr + 1, w, x, y);
+        bj_pair(0, X, sr, w, px, qx);
+        bj_pair(0, Y, sr, w, py, qy);
+        if (x == py || x == qy) {  // a pair is ordered by column
+          int o = X; X = Y; Y = o;
+          o = px; px = py; py = o;
+          o = qx; qx = qy; qy = o;
+        }
+        const float pp = G[px * kBJLd + py], pq = G[px * kBJLd + qy];
+        const float qp = G[qx * kBJLd + py], qq = G[qx * kBJLd + qy];
+        const float cx = __shfl_sync(all, cs, X), sx = __shfl_sync(all, sn, X);
+        const float cy = __shfl_sync(all, cs, Y), sy = __shfl_sync(all, sn, Y);
+        const float ax = __shfl_sync(all, an, X), bx = __shfl_sync(all, bn, X);
+        const float ay = __shfl_sync(all, an, Y), by = __shfl_sync(all, bn, Y);
+        const bool x2 = x == qx, y2 = y == qy;
+        const float ux = x2 ? sx : cx, vx = x2 ? cx : -sx, uy = y2 ? sy : cy, vy = y2 ? cy : -sy;
+        al = x2 ? bx : ax;
+        be = y2 ? by : ay;
+        ga = ux * (uy * pp + vy * pq) + vx * (uy * qp + vy * qq);
+      } else {
+        // x = column i, first of its pair before and after; y second of the next lane's pair
+        const float pp = G[i * kBJLd + Yc], pq = G[i * kBJLd + qy];
+        const float qp = G[qx * kBJLd + Yc], qq = G[qx * kBJLd + qy];
+        const float cy = __shfl_sync(all, cs, Yc), sy = __shfl_sync(all, sn, Yc);
+        be = __shfl_sync(all, bn, Yc);
+        al = an;
+        ga = cs * (sy * pp + cy * pq) - sn * (sy * qp + cy * qq);
+        qx = qx + 1 == w2 ? w : qx + 1;
+        qy = qy + 1 == w2 ? w : qy + 1;
+      }
+      bj_rotation(al, be, ga, nfloor, tol2, cs, sn, tn);
+      if (lane < w) s_rt[(sr + 1) & 1][lane] = make_float4(cs, sn, tn, ga);
+      bj_sub_barrier();
+    }
+    bj_sub_barrier();
+  } else if (warp >= 4 && warp < 12) {
+    const int e = tid - 128, a = e / w, b = e - a * w;
+    const bool on = e < w * w;
+    int pa = a, qa = w + a, pb = b, qb = w + b;
+    for (int sr = 0; sr < nsub; ++sr) {
+      if (on) {
+        if (kR0) {
+          bj_pair(0, a, sr, w, pa, qa);
+          bj_pair(0, b, sr, w, pb, qb);
+        }
+        const float4 ra = s_rt[sr & 1][a], rb = s_rt[sr & 1][b];
+        const float* G = Gs + ((sr & 1) ? kBJGs : 0);
+        float* Gn = Gs + ((sr & 1) ? 0 : kBJGs);
+        const int r0 = pa * kBJLd, r1 = qa * kBJLd;
+        const float pp = G[r0 + pb], pq = G[r0 + qb], qp = G[r1 + pb], qq = G[r1 + qb];
+        const float tpp = rb.x * pp - rb.y * pq, tpq = rb.y * pp + rb.x * pq;
+        const float tqp = rb.x * qp - rb.y * qq, tqq = rb.y * qp + rb.x * qq;
+        const bool dg = a == b;  // the norms carried through the rotation
+        const float off = ra.y != 0.f ? 0.f : pq;
+        Gn[r0 + pb] = dg ? fmaf(-ra.z, ra.w, pp) : ra.x * tpp - ra.y * tqp;
+        Gn[r0 + qb] = dg ? off : ra.x * tpq - ra.y * tqq;
+        Gn[r1 + pb] = dg ? off : ra.y * tpp + ra.x * tqp;
+        Gn[r1 + qb] = dg ? fmaf(ra.z, ra.w, qq) : ra.y * tpq + ra.x * tqq;
+        if (!kR0) {
+          qa = qa + 1 == w2 ? w : qa + 1;
+          qb = qb + 1 == w2 ? w : qb + 1;
+        }
+      }
+      bj_sub_barrier();
+    }
+  } else if (warp >= 12) {
+    const int e = tid - 384, nr = 128 / w, i0 = e / w, b = e - i0 * w;
+    const bool on = i0 < nr;
+    int pb = b, qb = w + b;
+    for (int sr = 0; sr < nsub; ++sr) {
+      if (on) {
+        if (kR0) bj_pair(0, b, sr, w, pb, qb);
+        const float4 rb = s_rt[sr & 1][b];
+        if (rb.y != 0.f) {
+          // at most four rows: 128 / w >= 8 of the 2w <= 32
+          float x[4], y[4];
+#pragma unroll
+          for (int k = 0; k < 4; ++k)
+            if (i0 + k * nr < w2) {
+              x[k] = Qs[(i0 + k * nr) * kBJLd + pb];
+              y[k] = Qs[(i0 + k * nr) * kBJLd + qb];
+            }
+#pragma unroll
+          for (int k = 0; k < 4; ++k)
+            if (i0 + k * nr < w2) {
+              Qs[(i0 + k * nr) * kBJLd + pb] = rb.x * x[k] - rb.y * y[k];
+              Qs[(i0 + k * nr) * kBJLd + qb] = rb.y * x[k] + rb.x * y[k];
+            }
+        }
+        if (!kR0) qb = qb + 1 == w2 ? w : qb + 1;
+      }
+      bj_sub_barrier();
+    }
+  }
+  __syncthreads();
+}
+
+// One round's pair work on the 2w <= 32 columns Ms [2w][rp] in shared memory:
+// the rotation Q (Qs [2w][kBJLd], set here) that the round applies to them.
+// Gs [2][kBJGs]: the Gram matrix [2w][kBJLd], twice.  Gi: null, or the Gram matrices
+// [2][w][w] of the two blocks (carried from where the blocks came from: then
+// only the cross products of a later round are formed).  Every thread of the
+// block calls it; null when nothing was rotated (Q = I, the Gram matrix in the
+// first copy), else the copy with the round's final Gram matrix.
+__device__ __forceinline__ const float* bj_round(int round, int w, int rp, const float* __restrict__ Ms,
+                                                 float* __restrict__ Qs, float* __restrict__ Gs,
+                                                 const float* __restrict__ Gi, float nfloor, float tol2) {
+  __shared__ float4 s_rt[2][16];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int w2 = 2 * w, rch = rp >> 2;
-  const bool resident = round > 0;  // column `warp` of block a lives in registers
-  float4 xr[NCH];
-  if (resident && warp < w) {
-    const float4* mp = reinterpret_cast<const float4*>(Ms + (size_t)warp * rp);
+  for (int i = warp; i < w2; i += kBJThreads / 32)
+    for (int j = lane; j < kBJLd; j += 32) Qs[i * kBJLd + j] = (i == j) ? 1.f : 0.f;
+  float v[16];
+  if (Gi != nullptr && round != 0) {
+    // the cross products, a warp per 4 x 4 tile (w <= 16: at most 16 tiles)
+    const int nt = (w + 3) >> 2, ta = warp / nt, tb = warp - ta * nt;
+    if (warp < nt * nt) {
+      bj_gram_tile<32>(Ms, rch, 4 * ta, w + 4 * tb, w - 1, w2 - 1, true, v);
+      const int ci = 4 * ta + ((lane & 15) >> 2), cj = 4 * tb + (lane & 3);
+      if (lane < 16 && ci < w && cj < w) {
+        Gs[ci * kBJLd + w + cj] = v[0];
+        Gs[(w + cj) * kBJLd + ci] = v[0];
+      }
+    }
+    for (int i = warp; i < w2; i += kBJThreads / 32) {
+      const int o = i < w ? 0 : w;
+      if (lane < w) Gs[i * kBJLd + o + lane] = Gi[i * w + lane];
+    }
+  } else {
+    // all of it by 4 x 4 tiles on and above the diagonal, four tiles a warp
+    const int ng = (w2 + 3) >> 2, ntile = ng * (ng + 1) / 2;
+    for (int t = warp * 4 + (lane >> 3); t - (lane >> 3) < ntile; t += (kBJThreads / 32) * 4) {
+      // tile (a, b), a <= b, column by column
+      const int b = ((int)sqrtf((float)(8 * t + 1)) - 1) >> 1;
+      const int a = t - b * (b + 1) / 2;
+      bj_gram_tile<8>(Ms, rch, 4 * a, 4 * b, w2 - 1, w2 - 1, t < ntile, v);
 #pragma unroll
-    for (int t = 0; t < NCH; ++t) {
-      const int c = lane + 32 * t;
-      xr[t] = c < rch ? mp[c] : make_float4(0.f, 0.f, 0.f, 0.f);
+      for (int u = 0; u < 2; ++u) {
+        const int e = 2 * (lane & 7) + u, ci = 4 * a + (e >> 2), cj = 4 * b + (e & 3);
+        if (t < ntile && cj < w2 && ci <= cj) {
+          Gs[ci * kBJLd + cj] = v[u];
+          Gs[cj * kBJLd + ci] = v[u];
+        }
+      }
     }
   }
-  const int nsub = (round == 0) ? w2 - 1 : w;
-  for (int sr = 0; sr < nsub; ++sr) {
-    // warp `warp` owns pair `warp` of the sub-round: inner product, its
-    // rotation (every lane computes it from the reduced sums), the update
-    // of the two columns, their tracked norms and Q's two columns; pairs
-    // of a sub-round are disjoint, so one barrier per sub-round suffices
-    if (warp < w) {
+  __syncthreads();
+  float al = 0.f, be = 0.f, ga = 0.f, cs = 1.f, sn = 0.f, tn = 0.f;  // warp 0: the lane's pair
+  {
+    auto over = [&](int p, int q) {
+      return bj_rotates(Gs[p * kBJLd + p], Gs[q * kBJLd + q], Gs[p * kBJLd + q], nfloor, tol2);
+    };
+    bool any = false;
+    const int e = tid & (kBJThreads / 2 - 1), a = e / w, b = e - a * w;
+    if (e < w * w) {
+      if (tid >= kBJThreads / 2)
+        any = over(a, w + b);
+      else if (round == 0 && a < b)
+        any = over(a, b) || over(w + a, w + b);
+    }
+    if (tid < w) {
       int p, q;
-      bj_pair(round, warp, sr, w, p, q);
-      float4 x[NCH], y[NCH];
-      const float4* mp = reinterpret_cast<const float4*>(Ms + (size_t)p * rp);
-      const float4* mq = reinterpret_cast<const float4*>(Ms + (size_t)q * rp);
-      float ga = 0.f;
-#pragma unroll
-      for (int t = 0; t < NCH; ++t) {
-        const int c = lane + 32 * t;
-        x[t] = resident ? xr[t] : (c < rch ? mp[c] : make_float4(0.f, 0.f, 0.f, 0.f));
-        y[t] = c < rch ? mq[c] : make_float4(0.f, 0.f, 0.f, 0.f);
-        ga = fmaf(x[t].x, y[t].x, ga);
-        ga = fmaf(x[t].y, y[t].y, ga);
-        ga = fmaf(x[t].z, y[t].z, ga);
-        ga = fmaf(x[t].w, y[t].w, ga);
-      }
-      ga = warp_sum(ga);
-      const float al = nrm[p], be = nrm[q];
-      const float fa = fmaxf(al, nfloor), fb = fmaxf(be, nfloor);
-      // rotate unless |g| <= tol |x| |y| (squared form; the block is scaled
-      // so that squared norms stay far from the FP32 range limits)
-      if (ga != 0.f && ga * ga > tol2 * fa * fb) {
-        // t the smaller root of t^2 + 2 zeta t - 1 = 0, zeta = (|y|^2 - |x|^2) / (2 g)
-        const float zeta = __fdividef(be - al, 2.f * ga);
-        const float az = fabsf(zeta);
-        float tt;
-        if (az > 1e18f) {
-          tt = __fdividef(0.5f, az);
-        } else {
-          const float s2 = fmaf(az, az, 1.f);
-          tt = __fdividef(1.f, az + s2 * rsqrtf(s2));
-        }
-        tt = copysignf(tt, zeta);
-        const float u = fmaf(tt, tt, 1.f);
-        float cs = rsqrtf(u);
-        cs = cs * fmaf(-0.5f * u, cs * cs, 1.5f);  // one Newton step: cs^2 (1 + t^2) = 1
-        const float sn = cs * tt;
-        float4* mpw = reinterpret_cast<float4*>(Ms + (size_t)p * rp);
-        float4* mqw = reinterpret_cast<float4*>(Ms + (size_t)q * rp);
-#pragma unroll
-        for (int t = 0; t < NCH; ++t) {
-          const int c = lane + 32 * t;
-          float4 a4, b4;
-          a4.x = cs * x[t].x - sn * y[t].x;
-          a4.y = cs * x[t].y - sn * y[t].y;
-          a4.z = cs * x[t].z - sn * y[t].z;
-          a4.w = cs * x[t].w - sn * y[t].w;
-          b4.x = sn * x[t].x + cs * y[t].x;
-          b4.y = sn * x[t].y + cs * y[t].y;
-          b4.z = sn * x[t].z + cs * y[t].z;
-          b4.w = sn * x[t].w + cs * y[t].w;
-          if (resident) xr[t] = a4;
-          else if (c < rch) mpw[c] = a4;
-          if (c < rch) mqw[c] = b4;
-        }
-        if (lane < w2) {
-          const float qp = Qs[lane * ldq + p], qq = Qs[lane * ldq + q];
-          Qs[lane * ldq + p] = cs * qp - sn * qq;
-          Qs[lane * ldq + q] = sn * qp + cs * qq;
-        }
-        if (lane == 0) {
-          nrm[p] = al - tt * ga;
-          nrm[q] = be + tt * ga;
-          *s_rot = 1;
-        }
-      }
+      bj_pair(round, tid, 0, w, p, q);
+      al = Gs[p * kBJLd + p];
+      be = Gs[q * kBJLd + q];
+      ga = Gs[p * kBJLd + q];
+      bj_rotation(al, be, ga, nfloor, tol2, cs, sn, tn);
+      s_rt[0][tid] = make_float4(cs, sn, tn, ga);
     }
-    __syncthreads();
+    if (!__syncthreads_or(any)) return nullptr;
   }
-  if (resident && warp < w) {
-    float4* mp = reinterpret_cast<float4*>(Ms + (size_t)warp * rp);
+  if (round == 0)
+    bj_subs<true>(w, Qs, Gs, s_rt, nfloor, tol2, al, be, ga, cs, sn, tn);
+  else
+    bj_subs<false>(w, Qs, Gs, s_rt, nfloor, tol2, al, be, ga, cs, sn, tn);
+  return Gs + (((round == 0 ? w2 - 1 : w) & 1) ? kBJGs : 0);
+}
+
+// Columns c0 .. c0 + 3 of X_blk Q for one 16-byte row chunk (X_blk [2w][ldx] in
+// shared memory), or of X_blk itself when the round rotated nothing; put(l,
+// values) takes column l < 2w.  Two columns per packed FMA.
+template <class Put>
+__device__ __forceinline__ void bj_apply(const float* __restrict__ X, int ldx, const float* __restrict__ Qs, int w2, int ch, int c0, bool rotated, Put put) {
+  if (!rotated) {
 #pragma unroll
-    for (int t = 0; t < NCH; ++t) {
-      const int c = lane + 32 * t;
-      if (c < rch) mp[c] = xr[t];
+    for (int j = 0; j < 4; ++j)
+      if (c0 + j < w2) put(c0 + j, reinterpret_cast<const float4*>(X + (size_t)(c0 + j) * ldx)[ch]);
+    return;
+  }
+  float2 acc[4][2];  // [row][column pair]
+#pragma unroll
+  for (int u = 0; u < 4; ++u)
+#pragma unroll
+    for (int j = 0; j < 2; ++j) acc[u][j] = make_float2(0.f, 0.f);
+  const float4* xp = reinterpret_cast<const float4*>(X) + ch;
+#pragma unroll 4
+  for (int k = 0; k < w2; ++k) {
+    const float4 v = xp[(size_t)k * (ldx >> 2)];
+    const float4 q = *reinterpret_cast<const float4*>(Qs + k * kBJLd + c0);
+    const float vv[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      acc[u][0] = fma2(make_float2(vv[u], vv[u]), make_float2(q.x, q.y), acc[u][0]);
+      acc[u][1] = fma2(make_float2(vv[u], vv[u]), make_float2(q.z, q.w), acc[u][1]);
+    }
+  }
+#pragma unroll
+  for (int j = 0; j < 2; ++j) {
+    if (c0 + 2 * j < w2) {  // 2w is even
+      put(c0 + 2 * j, make_float4(acc[0][j].x, acc[1][j].x, acc[2][j].x, acc[3][j].x));
+      put(c0 + 2 * j + 1, make_float4(acc[0][j].y, acc[1][j].y, acc[2][j].y, acc[3][j].y));
     }
   }
 }
 
 // Shared-memory layout: Ms [2w][rp] and Vs [2w][cp4] with rp, cp4 the row
-// counts rounded up to 4 (zero rows; float4 access), Qs [2w][ldq], nrm [2w].
-// NCH = row chunks of 4 per lane (rp <= 128 NCH).
-template <int NCH>
+// counts rounded up to 4 (zero rows; float4 access), Qs [2w][kBJLd], Gs.
 __global__ void __launch_bounds__(kBJThreads) k_block_jacobi(int r, int cpad, int w, float* __restrict__ M,
                                                              int ldm, float* __restrict__ V, int ldv,
                                                              float tol, int max_sweeps, int* __restrict__ rot,
@@ -916,86 +1173,51 @@ __global__ void __launch_bounds__(kBJThreads) k_block_jacobi(int r, int cpad, in
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int w2 = 2 * w;
   const int rp = (r + 3) & ~3, cp4 = (cpad + 3) & ~3;
-  const int ldq = (w2 + 7) & ~3;  // multiple of 4, >= 2w + 4
   float* Ms = reinterpret_cast<float*>(smem_raw);
   float* Vs = Ms + (size_t)w2 * rp;
   float* Qs = Vs + (size_t)w2 * cp4;
-  float* nrm = Qs + w2 * ldq;
+  float* Gs = Qs + w2 * kBJLd;
   const int P = gridDim.x, g = blockIdx.x, nblk = 2 * P;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = kBJThreads / 32;
   const float nfloor = floor_ptr ? *floor_ptr : 0.f;
   const float tol2 = tol * tol;
-  __shared__ int s_rot;
   int sweep = 0;
   for (; sweep < max_sweeps; ++sweep) {
-    if (tid == 0) s_rot = 0;
+    bool any_rot = false;  // the same in every thread of the CTA
     for (int round = 0; round < nblk - 1; ++round) {
       const int ba = (g == 0) ? 0 : 1 + add_mod(g - 1, round, nblk - 1);
       const int bb = 1 + add_mod(nblk - 2 - g, round, nblk - 1);
-      // load the 2w columns of M (with their squared norms) and of V; Q = I
+      // load the 2w columns of M and of V
       for (int l = warp; l < w2; l += nw) {
         const int gc = (l < w ? ba * w + l : bb * w + (l - w));
         const float* src = M + (size_t)gc * ldm;
         float* dst = Ms + (size_t)l * rp;
-        float s2 = 0.f;
-        for (int i = lane; i < rp; i += 32) {
-          const float v = i < r ? src[i] : 0.f;
-          dst[i] = v;
-          s2 = fmaf(v, v, s2);
-        }
-        s2 = warp_sum(s2);
-        if (lane == 0) nrm[l] = s2;
+        for (int i = lane; i < rp; i += 32) dst[i] = i < r ? src[i] : 0.f;
         const float* vsrc = V + (size_t)gc * ldv;
         float* vdst = Vs + (size_t)l * cp4;
         for (int i = lane; i < cp4; i += 32) vdst[i] = i < cpad ? vsrc[i] : 0.f;
       }
-      for (int e = tid; e < w2 * ldq; e += kBJThreads) {
-        const int i = e / ldq, j = e - i * ldq;
-        Qs[e] = (i == j) ? 1.f : 0.f;
-      }
       __syncthreads();
-      bj_round<NCH>(round, w, rp, Ms, Qs, ldq, nrm, nfloor, tol2, &s_rot);
-      __syncthreads();
-      // store back M
-      for (int l = warp; l < w2; l += nw) {
-        const int gc = (l < w ? ba * w + l : bb * w + (l - w));
-        const float* src = Ms + (size_t)l * rp;
-        float* dst = M + (size_t)gc * ldm;
-        for (int i = lane; i < r; i += 32) dst[i] = src[i];
-      }
-      // V_blk <- V_blk Q: thread = (float4 row chunk, 4 output columns)
-      {
-        const int vch = cp4 >> 2, ngrp = (w2 + 3) >> 2;
-        for (int e = tid; e < vch * ngrp; e += kBJThreads) {
-          const int ch = e % vch, c0 = (e / vch) * 4;
-          float4 acc[4];
-#pragma unroll
-          for (int j = 0; j < 4; ++j) acc[j] = make_float4(0.f, 0.f, 0.f, 0.f);
-          for (int k2 = 0; k2 < w2; ++k2) {
-            const float4 v = reinterpret_cast<const float4*>(Vs + (size_t)k2 * cp4)[ch];
-            const float4 qv = *reinterpret_cast<const float4*>(Qs + k2 * ldq + c0);
-            const float qq[4] = {qv.x, qv.y, qv.z, qv.w};
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-              acc[j].x = fmaf(v.x, qq[j], acc[j].x);
-              acc[j].y = fmaf(v.y, qq[j], acc[j].y);
-              acc[j].z = fmaf(v.z, qq[j], acc[j].z);
-              acc[j].w = fmaf(v.w, qq[j], acc[j].w);
-            }
+      const bool rotated = bj_round(round, w, rp, Ms, Qs, Gs, nullptr, nfloor, tol2) != nullptr;
+      any_rot |= rotated;
+      // M_blk Q and V_blk Q back: thread = (16-byte row chunk, 4 output columns)
+      if (rotated) {
+        const int ngrp = (w2 + 3) >> 2;
+        auto back = [&](const float* X, int ldx, float* out, int ldo, int rows) {
+          const int nch = ldx >> 2;
+          for (int e = tid; e < nch * ngrp; e += kBJThreads) {
+            const int ch = e % nch, c0 = (e / nch) * 4;
+            bj_apply(X, ldx, Qs, w2, ch, c0, true, [&](int l, float4 v) {
+              float* dst = out + (size_t)(l < w ? ba * w + l : bb * w + (l - w)) * ldo + 4 * ch;
+              if (4 * ch + 0 < rows) dst[0] = v.x;
+              if (4 * ch + 1 < rows) dst[1] = v.y;
+              if (4 * ch + 2 < rows) dst[2] = v.z;
+              if (4 * ch + 3 < rows) dst[3] = v.w;
+            });
           }
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            const int l = c0 + j;
-            if (l < w2) {
-              const int gc = (l < w ? ba * w + l : bb * w + (l - w));
-              float* dst = V + (size_t)gc * ldv + 4 * ch;
-              const float a4[4] = {acc[j].x, acc[j].y, acc[j].z, acc[j].w};
-#pragma unroll
-              for (int u = 0; u < 4; ++u)
-                if (4 * ch + u < cpad) dst[u] = a4[u];
-            }
-          }
-        }
+        };
+        back(Ms, rp, M, ldm, r);
+        back(Vs, cp4, V, ldv, cpad);
       }
       if (P > 1) {
         if (!grid_barrier(bar, P, err)) return;
@@ -1005,33 +1227,35 @@ __global__ void __launch_bounds__(kBJThreads) k_block_jacobi(int r, int cpad, in
     }
     // convergence test over the whole grid
     if (P > 1) {
-      if (tid == 0 && s_rot) atomicAdd(&rot[sweep], 1);
+      if (tid == 0 && any_rot) atomicAdd(&rot[sweep], 1);
       if (!grid_barrier(bar, P, err)) return;
       if (__ldcg(&rot[sweep]) == 0) break;
     } else {
-      __syncthreads();
-      if (!s_rot) break;
+      if (!any_rot) break;
     }
-    __syncthreads();
   }
   if (g == 0 && tid == 0 && sweeps_out) *sweeps_out = sweep;
 }
 
-// The same block Jacobi on one thread-block cluster (P <= 8 CTAs): the
-// columns stay in shared memory for the whole solve.  At the end of a round
-// each CTA sends its two blocks straight into the shared memory of the CTAs
-// that take them in the next round (double-buffered by round parity), the V
-// block as V_blk Q, so a round costs one cluster barrier and no global
-// traffic.  Shared memory: Mb [2][2w][rp], Vb [2][2w][cp4], Qs [2w][ldq],
-// nrm [2w].
-constexpr int kBJMaxCluster = 8;
+// The same block Jacobi on one thread-block cluster of 2P <= 16 CTAs: the
+// columns stay in shared memory for the whole solve.  CTA g < P works on block
+// pairs of M as above and sends its round's Q to CTA P + g, which holds the same
+// blocks of V and applies Q one round later, while the M side is on the next
+// round.  At the end of a round each CTA sends its two blocks straight into the
+// shared memory of the CTAs that take them in the next round (double-buffered
+// by round parity), as X_blk Q, so a round costs one cluster barrier and no
+// global traffic.  V on CTAs of its own takes half of the products and of the
+// exchange off a round's chain; the blocks' own Gram matrices travel with them
+// within a sweep.  Shared memory: Xb [2][2w][ldx] (M or V), Qs [2][2w][kBJLd]
+// (M: its own in the first; V: received, by round parity), Gs, Gi [2][2][w][w]
+// (received, by round parity).
+constexpr int kBJMaxCluster = 8;  // P
 
 __device__ __forceinline__ void bj_blocks(int g, int round, int nblk, int& ba, int& bb) {
   ba = (g == 0) ? 0 : 1 + add_mod(g - 1, round, nblk - 1);
   bb = 1 + add_mod(nblk - 2 - g, round, nblk - 1);
 }
 
-template <int NCH>
 __global__ void __launch_bounds__(kBJThreads) k_block_jacobi_cl(int r, int cpad, int w, float* __restrict__ M,
                                                                 int ldm, float* __restrict__ V, int ldv,
                                                                 float tol, int max_sweeps,
@@ -1040,16 +1264,20 @@ __global__ void __launch_bounds__(kBJThreads) k_block_jacobi_cl(int r, int cpad,
   namespace cg = cooperative_groups;
   cg::cluster_group cl = cg::this_cluster();
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int w2 = 2 * w;
-  const int rp = (r + 3) & ~3, cp4 = (cpad + 3) & ~3;
-  const int ldq = (w2 + 7) & ~3;
-  float* Mb = reinterpret_cast<float*>(smem_raw);
-  float* Vb = Mb + 2 * (size_t)w2 * rp;
-  float* Qs = Vb + 2 * (size_t)w2 * cp4;
-  float* nrm = Qs + w2 * ldq;
-  __shared__ int s_rot;
-  __shared__ int rotf[2][kBJMaxCluster];  // per-CTA "rotated" flags, by sweep parity
-  const int P = (int)cl.num_blocks(), g = (int)cl.block_rank(), nblk = 2 * P;
+  __shared__ int rotf[2][kBJMaxCluster];  // the M CTAs' "rotated" flags, by sweep parity
+  __shared__ int qrot[2];                 // V: whether the received Q rotates, by round parity
+  const int P = (int)cl.num_blocks() / 2, nblk = 2 * P;
+  const bool isv = (int)cl.block_rank() >= P;
+  const int first = isv ? P : 0, g = (int)cl.block_rank() - first;
+  const int w2 = 2 * w, rows = isv ? cpad : r, ldx = (rows + 3) & ~3, nch = ldx >> 2;
+  const int ngrp = (w2 + 3) >> 2, qsz = w2 * kBJLd;
+  const size_t xsz = (size_t)w2 * ((max(r, cpad) + 3) & ~3);  // one buffer, the same in every CTA
+  float* X0 = reinterpret_cast<float*>(smem_raw);
+  float* Q0 = X0 + 2 * xsz;
+  float* Gs = Q0 + 2 * qsz;
+  float* Gi = Gs + 2 * kBJGs;
+  float* X = isv ? V : M;
+  const int ldg = isv ? ldv : ldm;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = kBJThreads / 32;
   const float nfloor = floor_ptr ? *floor_ptr : 0.f;
   const float tol2 = tol * tol;
@@ -1057,121 +1285,99 @@ __global__ void __launch_bounds__(kBJThreads) k_block_jacobi_cl(int r, int cpad,
   bj_blocks(g, 0, nblk, ba, bb);
   // round 0's blocks into buffer 0
   for (int l = warp; l < w2; l += nw) {
-    const int gc = (l < w ? ba * w + l : bb * w + (l - w));
-    const float* src = M + (size_t)gc * ldm;
-    float* dst = Mb + (size_t)l * rp;
-    for (int i = lane; i < rp; i += 32) dst[i] = i < r ? src[i] : 0.f;
-    const float* vsrc = V + (size_t)gc * ldv;
-    float* vdst = Vb + (size_t)l * cp4;
-    for (int i = lane; i < cp4; i += 32) vdst[i] = i < cpad ? vsrc[i] : 0.f;
+    const float* src = X + (size_t)(l < w ? ba * w + l : bb * w + (l - w)) * ldg;
+    for (int i = lane; i < ldx; i += 32) X0[(size_t)l * ldx + i] = i < rows ? src[i] : 0.f;
   }
-  __syncthreads();
-  int buf = 0, sweep = 0;
+  cl.sync();  // every CTA of the cluster runs before the first remote write
+  // X_blk Q of the blocks of round `rd` in buffer `from` into the receivers'
+  // other buffer
+  auto send = [&](int rd, int from, const float* Qs, bool rotated, const float* Gf) {
+    const int nr = (rd + 1 == nblk - 1) ? 0 : rd + 1;
+    int mine[2], cta[2], slot[2];
+    bj_blocks(g, rd, nblk, mine[0], mine[1]);
+#pragma unroll
+    for (int s = 0; s < 2; ++s) {
+      cta[s] = 0;
+      slot[s] = 0;
+      for (int q = 0; q < P; ++q) {
+        int qa, qb;
+        bj_blocks(q, nr, nblk, qa, qb);
+        if (qa == mine[s]) { cta[s] = q; slot[s] = 0; }
+        if (qb == mine[s]) { cta[s] = q; slot[s] = 1; }
+      }
+    }
+    const float* Xs = X0 + (size_t)from * xsz;
+    float* Xn = X0 + (size_t)(from ^ 1) * xsz;
+    float* to[2];
+#pragma unroll
+    for (int s = 0; s < 2; ++s)
+      to[s] = cl.map_shared_rank(Xn + (size_t)slot[s] * w * ldx, first + cta[s]);
+    if (Gf != nullptr && nr != 0)
+#pragma unroll
+      for (int s = 0; s < 2; ++s) {
+        float* gi = cl.map_shared_rank(Gi + (2 * (from ^ 1) + slot[s]) * w * w, cta[s]);
+        for (int i = warp; i < w; i += nw)
+          if (lane < w) gi[i * w + lane] = Gf[(s * w + i) * kBJLd + s * w + lane];
+      }
+    for (int e = tid; e < nch * ngrp; e += kBJThreads) {
+      const int ch = e % nch, c0 = (e / nch) * 4;
+      bj_apply(Xs, ldx, Qs, w2, ch, c0, rotated, [&](int l, float4 v) {
+        const int s = l < w ? 0 : 1, li = l - s * w;
+        reinterpret_cast<float4*>((s ? to[1] : to[0]) + (size_t)li * ldx)[ch] = v;
+      });
+    }
+  };
+  int n = 0, sweep = 0;  // n: rounds begun; buffer n & 1 holds the round's blocks (V: the last round's, n - 1)
   for (; sweep < max_sweeps; ++sweep) {
-    if (tid == 0) s_rot = 0;
-    for (int round = 0; round < nblk - 1; ++round) {
-      bj_blocks(g, round, nblk, ba, bb);
-      float* Ms = Mb + (size_t)buf * w2 * rp;
-      float* Vs = Vb + (size_t)buf * w2 * cp4;
-      // squared norms of the 2w columns; Q = I
-      for (int l = warp; l < w2; l += nw) {
-        const float4* col = reinterpret_cast<const float4*>(Ms + (size_t)l * rp);
-        float s2 = 0.f;
-        for (int c = lane; c < (rp >> 2); c += 32) {
-          const float4 v = col[c];
-          s2 = fmaf(v.x, v.x, fmaf(v.y, v.y, fmaf(v.z, v.z, fmaf(v.w, v.w, s2))));
-        }
-        s2 = warp_sum(s2);
-        if (lane == 0) nrm[l] = s2;
+    bool any_rot = false;  // the same in every thread of the CTA
+    for (int round = 0; round < nblk - 1; ++round, ++n) {
+      if (!isv) {
+        const float* Gf = bj_round(round, w, ldx, X0 + (size_t)(n & 1) * xsz, Q0, Gs, Gi + 2 * (n & 1) * w * w,
+                                   nfloor, tol2);
+        const bool rotated = Gf != nullptr;
+        any_rot |= rotated;
+        float* Qv = cl.map_shared_rank(Q0 + (n & 1) * qsz, P + g);
+        if (rotated)
+          for (int e = tid; e < qsz / 4; e += kBJThreads)
+            reinterpret_cast<float4*>(Qv)[e] = reinterpret_cast<const float4*>(Q0)[e];
+        if (tid == 0) *cl.map_shared_rank(&qrot[n & 1], P + g) = rotated;
+        send(round, n & 1, Q0, rotated, rotated ? Gf : Gs);
+        if (round == nblk - 2 && tid < 2 * P) *cl.map_shared_rank(&rotf[sweep & 1][g], tid) = any_rot;
+      } else if (n > 0) {
+        const int q = (n - 1) & 1;
+        send(round == 0 ? nblk - 2 : round - 1, q, Q0 + q * qsz, qrot[q] != 0, nullptr);
       }
-      for (int e = tid; e < w2 * ldq; e += kBJThreads) {
-        const int i = e / ldq, j = e - i * ldq;
-        Qs[e] = (i == j) ? 1.f : 0.f;
-      }
-      __syncthreads();
-      bj_round<NCH>(round, w, rp, Ms, Qs, ldq, nrm, nfloor, tol2, &s_rot);
-      __syncthreads();
-      // where this CTA's blocks go next (round 0 of the next sweep after the last round)
-      const int nr = (round + 1 == nblk - 1) ? 0 : round + 1;
-      int dst_cta[2], dst_slot[2];
-      {
-        const int mine[2] = {ba, bb};
-        for (int s = 0; s < 2; ++s) {
-          dst_cta[s] = 0;
-          dst_slot[s] = 0;
-          for (int q = 0; q < P; ++q) {
-            int qa, qb;
-            bj_blocks(q, nr, nblk, qa, qb);
-            if (qa == mine[s]) { dst_cta[s] = q; dst_slot[s] = 0; }
-            if (qb == mine[s]) { dst_cta[s] = q; dst_slot[s] = 1; }
-          }
-        }
-      }
-      float* Mn = Mb + (size_t)(buf ^ 1) * w2 * rp;
-      float* Vn = Vb + (size_t)(buf ^ 1) * w2 * cp4;
-      // M columns: copy into the receivers' next buffer
-      {
-        const int rch = rp >> 2;
-        for (int e = tid; e < w2 * rch; e += kBJThreads) {
-          const int l = e / rch, ch = e - l * rch, s = l < w ? 0 : 1, li = l - s * w;
-          float4* dst = reinterpret_cast<float4*>(
-              cl.map_shared_rank(Mn + (size_t)(dst_slot[s] * w + li) * rp, dst_cta[s]));
-          dst[ch] = reinterpret_cast<const float4*>(Ms + (size_t)l * rp)[ch];
-        }
-      }
-      // V columns: V_blk Q into the receivers' next buffer
-      {
-        const int vch = cp4 >> 2, ngrp = (w2 + 3) >> 2;
-        for (int e = tid; e < vch * ngrp; e += kBJThreads) {
-          const int ch = e % vch, c0 = (e / vch) * 4;
-          float4 acc[4];
-#pragma unroll
-          for (int j = 0; j < 4; ++j) acc[j] = make_float4(0.f, 0.f, 0.f, 0.f);
-          for (int k2 = 0; k2 < w2; ++k2) {
-            const float4 v = reinterpret_cast<const float4*>(Vs + (size_t)k2 * cp4)[ch];
-            const float4 qv = *reinterpret_cast<const float4*>(Qs + k2 * ldq + c0);
-            const float qq[4] = {qv.x, qv.y, qv.z, qv.w};
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-              acc[j].x = fmaf(v.x, qq[j], acc[j].x);
-              acc[j].y = fmaf(v.y, qq[j], acc[j].y);
-              acc[j].z = fmaf(v.z, qq[j], acc[j].z);
-              acc[j].w = fmaf(v.w, qq[j], acc[j].w);
-            }
-          }
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            const int l = c0 + j;
-            if (l < w2) {
-              const int s = l < w ? 0 : 1, li = l - s * w;
-              float4* dst = reinterpret_cast<float4*>(
-                  cl.map_shared_rank(Vn + (size_t)(dst_slot[s] * w + li) * cp4, dst_cta[s]));
-              dst[ch] = acc[j];
-            }
-          }
-        }
-      }
-      if (round == nblk - 2 && tid < P) *cl.map_shared_rank(&rotf[sweep & 1][g], tid) = s_rot;
       cl.sync();
-      buf ^= 1;
     }
     int any = 0;
     for (int q = 0; q < P; ++q) any |= rotf[sweep & 1][q];
     if (!any) break;
   }
-  // the current buffer holds round 0's blocks
-  __syncthreads();
-  bj_blocks(g, 0, nblk, ba, bb);
-  const float* Ms = Mb + (size_t)buf * w2 * rp;
-  const float* Vs = Vb + (size_t)buf * w2 * cp4;
-  for (int l = warp; l < w2; l += nw) {
-    const int gc = (l < w ? ba * w + l : bb * w + (l - w));
-    float* dst = M + (size_t)gc * ldm;
-    for (int i = lane; i < r; i += 32) dst[i] = Ms[(size_t)l * rp + i];
-    float* vdst = V + (size_t)gc * ldv;
-    for (int i = lane; i < cpad; i += 32) vdst[i] = Vs[(size_t)l * cp4 + i];
+  // the last round's blocks: M's are in place for the next round 0; V's take
+  // the last Q on the way out
+  bj_blocks(g, isv ? nblk - 2 : 0, nblk, ba, bb);
+  if (isv) {
+    if (n > 0) {
+      const int q = (n - 1) & 1;
+      for (int e = tid; e < nch * ngrp; e += kBJThreads) {
+        const int ch = e % nch, c0 = (e / nch) * 4;
+        bj_apply(X0 + (size_t)q * xsz, ldx, Q0 + q * w2 * kBJLd, w2, ch, c0, qrot[q] != 0, [&](int l, float4 v) {
+          float* dst = X + (size_t)(l < w ? ba * w + l : bb * w + (l - w)) * ldg + 4 * ch;
+          if (4 * ch + 0 < rows) dst[0] = v.x;
+          if (4 * ch + 1 < rows) dst[1] = v.y;
+          if (4 * ch + 2 < rows) dst[2] = v.z;
+          if (4 * ch + 3 < rows) dst[3] = v.w;
+        });
+      }
+    }
+  } else {
+    const float* Xs = X0 + (size_t)(n & 1) * xsz;
+    for (int l = warp; l < w2; l += nw) {
+      float* dst = X + (size_t)(l < w ? ba * w + l : bb * w + (l - w)) * ldg;
+      for (int i = lane; i < rows; i += 32) dst[i] = Xs[(size_t)l * ldx + i];
+    }
+    if (g == 0 && tid == 0 && sweeps_out) *sweeps_out = sweep;
   }
-  if (g == 0 && tid == 0 && sweeps_out) *sweeps_out = sweep;
 }
 
 // identity (cpad x cpad) and copy/convert of an r x c matrix into an r x cpad
@@ -1476,14 +1682,12 @@ __global__ void k_colnorm_floor(int r, int c, const T* __restrict__ M, int ldm, 
 
 static size_t bj_smem(int r, int cpad, int w) {
   const size_t rp = (r + 3) & ~3, cp4 = (cpad + 3) & ~3;
-  const size_t ldq = (2 * w + 7) & ~3;
-  return ((size_t)2 * w * (rp + cp4) + (size_t)2 * w * ldq + 2 * (size_t)w) * sizeof(float);
+  return ((size_t)2 * w * (rp + cp4) + (size_t)2 * w * kBJLd + 2 * kBJGs) * sizeof(float);
 }
 
 static size_t bj_cl_smem(int r, int cpad, int w) {
   const size_t rp = (r + 3) & ~3, cp4 = (cpad + 3) & ~3;
-  const size_t ldq = (2 * w + 7) & ~3;
-  return ((size_t)4 * w * (rp + cp4) + (size_t)2 * w * ldq + 2 * (size_t)w) * sizeof(float);
+  return ((size_t)4 * w * (rp > cp4 ? rp : cp4) + (size_t)4 * w * kBJLd + 2 * kBJGs + (size_t)4 * w * w) * sizeof(float);
 }
 
 static rr_status launch_bj(cudaStream_t s, int r, int cpad, int w, int P, float* M, float* V, float tol,
@@ -1493,34 +1697,35 @@ static rr_status launch_bj(cudaStream_t s, int r, int cpad, int w, int P, float*
   const size_t csm = bj_cl_smem(r, cpad, w);
   if (P <= kBJMaxCluster && csm <= 220 * 1024) {
     // one cluster: columns stay in shared memory, no global barrier
-    const void* fn = rp <= 128 ? (const void*)k_block_jacobi_cl<1>
-                     : rp <= 256 ? (const void*)k_block_jacobi_cl<2>
-                                 : (const void*)k_block_jacobi_cl<3>;
+    const void* fn = (const void*)k_block_jacobi_cl;
     if (csm > 48 * 1024)
       RR_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)csm));
+    if (2 * P > 8) RR_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(P);
+    cfg.gridDim = dim3(2 * P);
     cfg.blockDim = dim3(kBJThreads);
     cfg.dynamicSmemBytes = csm;
     cfg.stream = s;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = P;
+    at[0].val.clusterDim.x = 2 * P;
     at[0].val.clusterDim.y = 1;
     at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    int ld = r, ldv = cpad;
-    int* sw = ws.sweeps;
-    void* args[] = {&r, &cpad, &w, &M, &ld, &V, &ldv, &tol, &max_sweeps, &sw, &floor_ptr};
-    RR_CUDA(cudaLaunchKernelExC(&cfg, fn, args));
-    note_launches(1);
-    return RR_OK;
+    int nc = 0;
+    if (cudaOccupancyMaxActiveClusters(&nc, fn, &cfg) == cudaSuccess && nc >= 1) {
+      int ld = r, ldv = cpad;
+      int* sw = ws.sweeps;
+      void* args[] = {&r, &cpad, &w, &M, &ld, &V, &ldv, &tol, &max_sweeps, &sw, &floor_ptr};
+      RR_CUDA(cudaLaunchKernelExC(&cfg, fn, args));
+      note_launches(1);
+      return RR_OK;
+    }
+    (void)cudaGetLastError();
   }
   const size_t smem = bj_smem(r, cpad, w);
-  const void* fn = rp <= 128 ? (const void*)k_block_jacobi<1>
-                   : rp <= 256 ? (const void*)k_block_jacobi<2>
-                               : (const void*)k_block_jacobi<3>;
+  const void* fn = (const void*)k_block_jacobi;
   if (smem > 48 * 1024)
     RR_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   RR_CUDA(cudaMemsetAsync(ws.rot, 0, 64 * sizeof(int), s));
