@@ -379,31 +379,42 @@ __global__ void k_zero_dropped(int b1, int b2, double* __restrict__ C, const int
 
 // Column norms sigma_j of M (r x c), descending order with ties by index;
 // zero columns (dropped directions) sort last and are flagged invalid.
-__global__ void __launch_bounds__(kSmallThreads) k_colnorm_sort(int r, int c, const double* __restrict__ M,
-                                                                int ldm, double* __restrict__ sig,
-                                                                int* __restrict__ order) {
-  extern __shared__ double sh[];
-  double* nrm = sh;  // [c]
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  for (int j = warp; j < c; j += kSmallThreads / 32) {
-    double s = 0.0;
-    for (int i = lane; i < r; i += 32) s = fma(M[i + j * ldm], M[i + j * ldm], s);
-    s = warp_sum(s);
-    if (lane == 0) nrm[j] = sqrt(s);
-  }
-  __syncthreads();
+__global__ void __launch_bounds__(256) k_colnorms(int r, int c, const double* __restrict__ M, int ldm,
+                                                  double* __restrict__ sig) {
+  const int lane = threadIdx.x & 31, j = blockIdx.x * 8 + (threadIdx.x >> 5);
+  if (j >= c) return;
+  double s = 0.0;
+  for (int i = lane; i < r; i += 32) s = fma(M[i + (size_t)j * ldm], M[i + (size_t)j * ldm], s);
+  s = warp_sum(s);
+  if (lane == 0) sig[j] = sqrt(s);
+}
+
+__global__ void __launch_bounds__(kSmallThreads) k_norm_sort(int c, double* __restrict__ sig,
+                                                             int* __restrict__ order) {
+  extern __shared__ long long key[];  // [c]
+  const int tid = threadIdx.x;
   // a total order (a NaN norm counts as -1: last, flagged invalid with 0), so
-  // the ranks form a permutation whatever the data
+  // the ranks form a permutation whatever the data; nonnegative doubles order
+  // as their bits
+  for (int j = tid; j < c; j += kSmallThreads) key[j] = sig[j] >= 0.0 ? __double_as_longlong(sig[j]) : -1ll;
+  __syncthreads();
   for (int j = tid; j < c; j += kSmallThreads) {
-    const double v = nrm[j] >= 0.0 ? nrm[j] : -1.0;
+    const long long v = key[j];
     int rank = 0;
-    for (int l = 0; l < c; ++l) {
-      const double w = nrm[l] >= 0.0 ? nrm[l] : -1.0;
-      if (w > v || (w == v && l < j)) ++rank;
-    }
+    for (int l = 0; l < c; ++l) rank += key[l] > v || (key[l] == v && l < j);
     order[rank] = j;
-    sig[rank] = v >= 0.0 ? v : 0.0;
+    sig[rank] = v >= 0 ? __longlong_as_double(v) : 0.0;
   }
+}
+
+// Column norms of M (r x c) in descending order and where they came from.  The
+// norms on as many CTAs as columns ask for and the ranks from integer keys: both
+// are bound by the two FP64 operations a clock of one SM otherwise (105 -> 11
+// us at 256 columns).
+static void colnorm_sort(cudaStream_t s, int r, int c, const double* M, int ldm, double* sig, int* order) {
+  k_colnorms<<<(c + 7) / 8, 256, 0, s>>>(r, c, M, ldm, sig);
+  k_norm_sort<<<1, kSmallThreads, c * sizeof(long long), s>>>(c, sig, order);
+  note_launches(1);  // the caller counts the other
 }
 
 // Eigen finish: theta_rank = sigma + mu for valid columns, ascending order;
@@ -1384,16 +1395,28 @@ __global__ void __launch_bounds__(kBJThreads) k_block_jacobi_cl(int r, int cpad,
 // padded one (zero padding columns)
 // Power of two 2^-e with 2^(e-1) <= max |A| < 2^e (1 for a zero matrix), one block.
 __global__ void k_pow2_scale(int r, int c, const double* __restrict__ A, int lda, float* __restrict__ out) {
-  __shared__ double red[32];
-  double m = 0.0;
+  // magnitudes compare as their bits (an integer maximum: the FP64 one of 65536
+  // entries costs one SM 17 us more); a NaN is passed over
+  using u64 = unsigned long long;
+  constexpr u64 kInf = 0x7ff0000000000000ull;
+  __shared__ u64 red[32];
+  u64 m = 0;
   for (int j = threadIdx.x >> 5; j < c; j += blockDim.x >> 5)
-    for (int i = threadIdx.x & 31; i < r; i += 32) m = fmax(m, fabs(A[i + (size_t)j * lda]));
-  m = warp_max(m);
+#pragma unroll 4
+    for (int i = threadIdx.x & 31; i < r; i += 32) {
+      const u64 v = (u64)__double_as_longlong(A[i + (size_t)j * lda]) & ~(1ull << 63);
+      m = v <= kInf && v > m ? v : m;
+    }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const u64 v = __shfl_xor_sync(0xffffffffu, m, o);
+    m = v > m ? v : m;
+  }
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
   __syncthreads();
   if (threadIdx.x == 0) {
-    double v = 0.0;
-    for (int k = 0; k < (int)(blockDim.x >> 5); ++k) v = fmax(v, red[k]);
+    for (int k = 0; k < (int)(blockDim.x >> 5); ++k) m = red[k] > m ? red[k] : m;
+    const double v = __longlong_as_double((long long)m);
     int e = 0;
     if (v > 0.0) frexp(v, &e);
     *out = (float)ldexp(1.0, -e);
@@ -1516,21 +1539,34 @@ static bool carve_pencil(Arena& ar, int b1, int b2, PencilWs& w) {
 // Each factor is at most the matching extreme eigenvalue and at least 1/b of
 // it, so out lies in [cond_2(G) / b^2, cond_2(G)].  Also writes the number
 // of dropped columns (drop flags) to out[2].  One block.
-__global__ void k_cond_est(int b, const double* __restrict__ G, const double* __restrict__ W,
-                           const int* __restrict__ drop, double* __restrict__ out) {
-  __shared__ double sg[32], sw[32];
+__global__ void __launch_bounds__(1024) k_cond_est(int b, const double* __restrict__ G,
+                                                   const double* __restrict__ W, const int* __restrict__ drop,
+                                                   double* __restrict__ out) {
+  // four threads per row of W (their column ranges summed through shared
+  // memory), so that the loads of a row are not one chain
+  __shared__ double sg[32], sw[32], part[4][256];
   __shared__ int sd[32];
   double mg = 0.0, mw = 0.0;
   int nd = 0;
-  for (int i = threadIdx.x; i < b; i += blockDim.x) {
-    nd += drop[i] != 0;
-    mg = fmax(mg, G[i + (size_t)i * b]);
+  const int row = threadIdx.x & 255, q = threadIdx.x >> 8;
+  for (int i0 = 0; i0 < b; i0 += 256) {
+    const int i = i0 + row;
     double acc = 0.0;
-    for (int j = 0; j < b; ++j) {
-      const double w = W[i + (size_t)j * b];
-      acc = fma(w, w, acc);
+    if (i < b) {
+#pragma unroll 8
+      for (int j = q; j < b; j += 4) {
+        const double w = W[i + (size_t)j * b];
+        acc = fma(w, w, acc);
+      }
     }
-    mw = fmax(mw, acc);
+    part[q][row] = acc;
+    __syncthreads();
+    if (q == 0 && i < b) {
+      nd += drop[i] != 0;
+      mg = fmax(mg, G[i + (size_t)i * b]);
+      mw = fmax(mw, (part[0][row] + part[1][row]) + (part[2][row] + part[3][row]));
+    }
+    __syncthreads();
   }
   mg = warp_max(mg);
   mw = warp_max(mw);
@@ -1778,10 +1814,6 @@ struct QrCand {
   float tau, beta;
 };
 
-__device__ __forceinline__ bool qr_better(float n, int k, float bn, int bk) {
-  return n > bn || (n == bn && k < bk);
-}
-
 // Warp sums of N (a power of two <= 32) per-lane values at once
 // (reduce-scatter: halving exchanges over the top lane bits, then butterflies
 // over the rest): on return lane l holds the sum of value l >> (5 - log2 N).
@@ -1826,13 +1858,12 @@ __global__ void __launch_bounds__(kQrThreads, 1)
   cg::cluster_group cl = cg::this_cluster();
   __shared__ __align__(16) float vbuf[2][kQrMaxNC][kQrMaxRows];
   __shared__ QrCand cand[2][kQrMaxNC];
-  __shared__ unsigned long long s_key[2];
+  __shared__ unsigned long long s_key[kQrWarps];
   const int NC = (int)cl.num_blocks();
   const int z = (int)cl.block_rank();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const float sc = *scale;
   const int col0 = z * kQrWarps * CPW + warp;  // column of slot u: col0 + 16 u
-  if (threadIdx.x < 2) s_key[threadIdx.x] = 0ull;
 
   float a[CPW][RPL];
   unsigned done = 0;  // slot u pivoted already (or beyond the last column)
@@ -1867,10 +1898,14 @@ __global__ void __launch_bounds__(kQrThreads, 1)
     const unsigned hi = (unsigned)(key >> 32), lo = (unsigned)key;
     const unsigned mhi = __reduce_max_sync(0xffffffffu, hi);
     const unsigned mlo = __reduce_max_sync(0xffffffffu, hi == mhi ? lo : 0u);
-    const unsigned long long wk = ((unsigned long long)mhi << 32) | mlo;
-    if (lane == 0 && wk) atomicMax(&s_key[par], wk);
+    // every warp's best, then every warp the best of them (filled again only
+    // after the next cluster barrier)
+    if (lane == 0) s_key[warp] = ((unsigned long long)mhi << 32) | mlo;
     __syncthreads();
-    const unsigned long long bk = s_key[par];
+    const unsigned long long wk = lane < kQrWarps ? s_key[lane] : 0ull;
+    const unsigned bhi = __reduce_max_sync(0xffffffffu, (unsigned)(wk >> 32));
+    const unsigned blo = __reduce_max_sync(0xffffffffu, (unsigned)(wk >> 32) == bhi ? (unsigned)wk : 0u);
+    const unsigned long long bk = ((unsigned long long)bhi << 32) | blo;
     if (bk == 0ull) {  // every column of this CTA is pivoted: publish "none"
       if (threadIdx.x < NC) {
         QrCand* dst = cl.map_shared_rank(&cand[par][z], (int)threadIdx.x);
@@ -1908,7 +1943,8 @@ __global__ void __launch_bounds__(kQrThreads, 1)
     for (int q = 0; q < NC; ++q) {
       float* dst = cl.map_shared_rank(&vbuf[par][z][0], q);
 #pragma unroll
-      for (int t = 0; t < RPL; ++t) dst[t * 32 + lane] = x[t];
+      for (int t = 0; t < RPL; ++t)
+        if (t * 32 + 31 >= j1) dst[t * 32 + lane] = x[t];  // rows < j1 are zero: not read
       if (lane == 0) *cl.map_shared_rank(&cand[par][z], q) = QrCand{cn, ck, tau, beta};
     }
   };
@@ -1917,27 +1953,23 @@ __global__ void __launch_bounds__(kQrThreads, 1)
   for (int j = 0; j < c; ++j) {
     cl.sync();
     const int par = j & 1;
-    // the key publish(j - 1) filled (read before this step's cluster barrier;
-    // filled next by publish(j + 1), after the next one)
-    if (threadIdx.x == 0) s_key[par] = 0ull;
-    QrCand b = cand[par][0];
-    int zs = 0;
-    for (int q = 1; q < NC; ++q) {
-      const QrCand m = cand[par][q];
-      if (qr_better(m.nrm2, m.col, b.nrm2, b.col)) {
-        b = m;
-        zs = q;
-      }
-    }
+    // the largest norm's candidate, lane = CTA; ties to the lower column
+    const QrCand m = lane < NC ? cand[par][lane] : QrCand{-1.f, INT_MAX, 0.f, 0.f};
+    const unsigned mh = m.col != INT_MAX ? __float_as_uint(m.nrm2) + 1u : 0u;
+    const unsigned bh = __reduce_max_sync(0xffffffffu, mh);
+    const unsigned bl = __reduce_max_sync(0xffffffffu, mh == bh ? ~(unsigned)m.col : 0u);
+    const int zs = __ffs(__ballot_sync(0xffffffffu, mh == bh && ~(unsigned)m.col == bl)) - 1;
+    const int bcol = (int)~bl;
+    const float btau = __shfl_sync(0xffffffffu, m.tau, zs), bbeta = __shfl_sync(0xffffffffu, m.beta, zs);
     const float* v = &vbuf[par][zs][0];
     float vr[RPL];
 #pragma unroll
-    for (int t = 0; t < RPL; ++t) vr[t] = v[t * 32 + lane];
+    for (int t = 0; t < RPL; ++t) vr[t] = t * 32 + lane >= j ? v[t * 32 + lane] : 0.f;
     if (z == j % NC) {
-      for (int i = threadIdx.x; i < c; i += kQrThreads) Hv[(size_t)j * c + i] = v[i];
-      if (threadIdx.x == 0) tq[j] = b.tau;
+      for (int i = threadIdx.x; i < c; i += kQrThreads) Hv[(size_t)j * c + i] = i >= j ? v[i] : 0.f;
+      if (threadIdx.x == 0) tq[j] = btau;
     }
-    // w_u = tau v^T a_u for the warp's 8 columns at once, then a_u -= w_u v
+    // w_u = tau v^T a_u for the warp's columns at once, then a_u -= w_u v
     // (pivoted columns have zero entries at rows >= j: no change)
     float d[CPW];
 #pragma unroll
@@ -1947,16 +1979,16 @@ __global__ void __launch_bounds__(kQrThreads, 1)
       for (int t = 0; t < RPL; ++t) s2 = fmaf(vr[t], a[u][t], s2);
       d[u] = s2;
     }
-    const float wsum = qr_rs<CPW>(d) * b.tau;
+    const float wsum = qr_rs<CPW>(d) * btau;
 #pragma unroll
     for (int u = 0; u < CPW; ++u) {
       const float wu = __shfl_sync(0xffffffffu, wsum, qr_rs_lane<CPW>(u));
       const int k = col0 + kQrWarps * u;
-      if (k == b.col) {  // the pivot column becomes beta e_j
+      if (k == bcol) {  // the pivot column becomes beta e_j
 #pragma unroll
         for (int t = 0; t < RPL; ++t) {
           const int i = t * 32 + lane;
-          a[u][t] = i == j ? b.beta : (i > j ? 0.f : a[u][t]);
+          a[u][t] = i == j ? bbeta : (i > j ? 0.f : a[u][t]);
         }
         done |= 1u << u;
       } else if (!((done >> u) & 1u)) {
@@ -2057,8 +2089,10 @@ static bool qr_precond_applies(int r, int c) { return r >= c && c >= kQrMinCols 
 
 static rr_status launch_qr_precond(cudaStream_t s, int r, int c, const double* C, const float* scale, float* X,
                                    int cpad, float* V, float* Hv, float* tq) {
-  const int rpl = c <= 128 ? 4 : c <= 256 ? 8 : 12;
-  const int cpw = rpl <= 8 ? 8 : 4;
+  // two columns a warp while that fits the cluster (256 columns of C^T on 8
+  // CTAs): at 256 x 256, with a shared-memory atomic per warp for the pivot and
+  // whole reflectors sent, 16 x 8 columns a CTA took 852 us, this 526
+  const int cpw = r <= 2 * kQrWarps * kQrMaxNC ? 2 : 4;
   const int NC = (r + kQrWarps * cpw - 1) / (kQrWarps * cpw);
   if (c > r || c > kQrMaxRows || NC > kQrMaxNC || cpad < c) return RR_ERR_ARG;
   cudaLaunchConfig_t cfg = {};
@@ -2073,10 +2107,10 @@ static rr_status launch_qr_precond(cudaStream_t s, int r, int c, const double* C
   at[0].val.clusterDim.z = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  if (rpl == 4)
-    RR_CUDA(cudaLaunchKernelEx(&cfg, k_qr_precond<4, 8>, r, c, C, scale, X, cpad, V, Hv, tq));
-  else if (rpl == 8)
-    RR_CUDA(cudaLaunchKernelEx(&cfg, k_qr_precond<8, 8>, r, c, C, scale, X, cpad, V, Hv, tq));
+  if (cpw == 2)
+    RR_CUDA(cudaLaunchKernelEx(&cfg, k_qr_precond<8, 2>, r, c, C, scale, X, cpad, V, Hv, tq));
+  else if (c <= 256)
+    RR_CUDA(cudaLaunchKernelEx(&cfg, k_qr_precond<8, 4>, r, c, C, scale, X, cpad, V, Hv, tq));
   else
     RR_CUDA(cudaLaunchKernelEx(&cfg, k_qr_precond<12, 4>, r, c, C, scale, X, cpad, V, Hv, tq));
   note_launches(1);
@@ -2438,13 +2472,13 @@ extern "C" rr_status rr_pencil_eig(int64_t b, const double* H, const double* G, 
   RR_CUDA(cudaMemsetAsync(w.err, 0, sizeof(int), s));
   whiten(s, n, G, WhitenScratch{w.W1, w.W2, w.T, w.E, w.E2, w.F}, w.drop1, w.W1);
   RR_CUDA(cudaMemsetAsync(w.cond, 0, 4 * sizeof(double), s));
-  k_cond_est<<<1, 256, 0, s>>>(n, G, w.W1, w.drop1, w.cond);
+  k_cond_est<<<1, 1024, 0, s>>>(n, G, w.W1, w.drop1, w.cond);
   // C = W^T H W, symmetrised and shifted positive definite (C - mu I)
   gemm_small(s, 0, 0, n, n, n, 1.0, H, n, w.W1, n, 0.0, w.T, n);
   gemm_small_sym(s, n, n, w.W1, n, w.T, n, w.C, n);  // W^T H W (symmetric)
   RR_TRY(eig_shift(s, n, w.C, w.drop1, w.sh, w.shok, w.mu));
   RR_TRY(jacobi_svd(s, n, n, w.C, w, w.M, w.V));
-  k_colnorm_sort<<<1, kSmallThreads, n * sizeof(double), s>>>(n, n, w.M, n, w.sig, w.order);
+  colnorm_sort(s, n, n, w.M, n, w.sig, w.order);
   k_eig_finish<<<1, 256, 0, s>>>(n, w.sig, w.order, w.mu, w.V, theta, w.T, w.nvalid);
   // Y = W Z
   gemm_small(s, 0, 0, n, n, n, 1.0, w.W1, n, w.T, n, 0.0, Y, n);
@@ -2477,18 +2511,18 @@ extern "C" rr_status rr_pencil_svd(int64_t b1, int64_t b2, const double* B, cons
   RR_CUDA(cudaStreamWaitEvent(ss.s2, ss.fork, 0));
   whiten(s, n1, Gu, WhitenScratch{w.W1, w.W2, w.T, w.E, w.E2, w.F}, w.drop1, w.C);
   whiten(ss.s2, n2, Gv, w.wb, w.drop2, w.V);
-  k_cond_est<<<1, 256, 0, ss.s2>>>(n2, Gv, w.V, w.drop2, w.cond + 1);  // cond[1], drops[3]
+  k_cond_est<<<1, 1024, 0, ss.s2>>>(n2, Gv, w.V, w.drop2, w.cond + 1);  // cond[1], drops[3]
   RR_CUDA(cudaEventRecord(ss.join, ss.s2));
   RR_CUDA(cudaStreamWaitEvent(s, ss.join, 0));
   RR_CUDA(cudaMemcpyAsync(w.W1, w.C, (size_t)n1 * n1 * sizeof(double), cudaMemcpyDeviceToDevice, s));
   RR_CUDA(cudaMemcpyAsync(w.W2, w.V, (size_t)n2 * n2 * sizeof(double), cudaMemcpyDeviceToDevice, s));
-  k_cond_est<<<1, 256, 0, s>>>(n1, Gu, w.W1, w.drop1, w.cond);      // cond[0], drops[2]
+  k_cond_est<<<1, 1024, 0, s>>>(n1, Gu, w.W1, w.drop1, w.cond);      // cond[0], drops[2]
   // Cw = Wu^T B Wv (b1 x b2) -> C
   gemm_small(s, 0, 0, n1, n2, n2, 1.0, B, n1, w.W2, n2, 0.0, w.T, n1);
   gemm_small(s, 1, 0, n1, n2, n1, 1.0, w.W1, n1, w.T, n1, 0.0, w.C, n1);
   k_zero_dropped<<<(n1 * n2 + 255) / 256, 256, 0, s>>>(n1, n2, w.C, w.drop1, w.drop2);
   RR_TRY(jacobi_svd(s, n1, n2, w.C, w, w.M, w.V));   // M = Cw V (b1 x b2), V (b2 x b2)
-  k_colnorm_sort<<<1, kSmallThreads, n2 * sizeof(double), s>>>(n1, n2, w.M, n1, w.sig, w.order);
+  colnorm_sort(s, n1, n2, w.M, n1, w.sig, w.order);
   double* Uw = w.T;   // b1 x r
   double* Vw = w.E;   // b2 x r
   k_svd_finish<<<64, 256, 0, s>>>(n1, n2, w.sig, w.order, w.M, w.V, sv, Uw, Vw, r);
