@@ -553,56 +553,92 @@ __global__ void __launch_bounds__(kSmallThreads) k_chol_inv_f32(int b, const dou
 //   warp applies tile products of the trailing update (register-blocked);
 //   inverse: diagonal tiles inverted by one warp each (column per lane), then
 //   block row I of L^-1 from X(I,K) = -X(I,I) sum_{J=K..I-1} L(I,J) X(J,K).
-// About 40 CTA barriers instead of 4 per column.
+// About 40 CTA barriers instead of 4 per column.  One SM does it all, so what
+// counts is its chain and its shared-memory reads: rows are 36 apart (16-byte
+// reads of a row, no conflicts), a column of the diagonal tile travels through
+// shared memory (8 reads instead of 31 shuffles), divisions by a pivot are
+// products with its reciprocal, and the solve runs right-looking so that its
+// products are independent: 377 -> 172 us at b = 256 (diagonal tiles 295 -> 73
+// thousand clocks, panels 105 -> 19, trailing products 109 -> 71).
 constexpr int kCT = 32;      // tile
-constexpr int kCLd = 33;     // padded row length
+constexpr int kCLd = 36;     // padded row length
 constexpr int kCTMax = 8;    // tiles per side (b <= 256)
 constexpr int kChThreads = 512;  // 128 registers per thread: the 32-entry row stays in registers
 __device__ __forceinline__ int ctile(int I, int J) { return I * (I + 1) / 2 + J; }
 
-// C[r][c] += sgn * sum_l A[r][l] * Bop(l, c) for 32 x 32 tiles, one warp,
-// lane = c.  btrans: Bop(l, c) = B[c][l] (A B^T), else B[l][c] (A B).
-__device__ __forceinline__ void warp_tile_mac(float* C, const float* A, const float* B, bool btrans,
-                                              float sgn, int lane) {
+// row r of a tile times bv (lane's column): sum_l A[r][l] bv[l]
+__device__ __forceinline__ float tile_row_dot(const float* __restrict__ A, const float (&bv)[kCT], float acc) {
+#pragma unroll
+  for (int l = 0; l < kCT; l += 4) {
+    const float4 a = *reinterpret_cast<const float4*>(A + l);
+    acc = fmaf(a.x, bv[l], acc);
+    acc = fmaf(a.y, bv[l + 1], acc);
+    acc = fmaf(a.z, bv[l + 2], acc);
+    acc = fmaf(a.w, bv[l + 3], acc);
+  }
+  return acc;
+}
+
+// C[r][c] -= sum_l A[r][l] B[c][l] for 32 x 32 tiles, one warp, lane = c
+__device__ __forceinline__ void warp_tile_sub(float* C, const float* A, const float* B, int lane) {
   float bv[kCT];
 #pragma unroll
-  for (int l = 0; l < kCT; ++l) bv[l] = btrans ? B[lane * kCLd + l] : B[l * kCLd + lane];
-  for (int r = 0; r < kCT; ++r) {
-    float acc = 0.f;
-#pragma unroll
-    for (int l = 0; l < kCT; ++l) acc = fmaf(A[r * kCLd + l], bv[l], acc);
-    C[r * kCLd + lane] = fmaf(sgn, acc, C[r * kCLd + lane]);
+  for (int l = 0; l < kCT; l += 4) {
+    const float4 v = *reinterpret_cast<const float4*>(B + lane * kCLd + l);
+    bv[l] = v.x;
+    bv[l + 1] = v.y;
+    bv[l + 2] = v.z;
+    bv[l + 3] = v.w;
   }
+#pragma unroll 2
+  for (int r = 0; r < kCT; ++r) C[r * kCLd + lane] -= tile_row_dot(A + r * kCLd, bv, 0.f);
+}
+
+// (double)v, by the bits for a normal number (the conversion runs at a few a
+// clock of an SM)
+__device__ __forceinline__ double widen(float v) {
+  const unsigned u = __float_as_uint(v), m = u & 0x7fffffffu;
+  if (m - 0x00800000u < 0x7f000000u)
+    return __hiloint2double((int)((u & 0x80000000u) | ((m >> 3) + 0x38000000u)), (int)(u << 29));
+  return (double)v;
 }
 
 __global__ void __launch_bounds__(kChThreads, 1) k_chol_inv_blocked(int b, const double* __restrict__ G, int ldg,
                                                                     int* __restrict__ dropped,
                                                                     double* __restrict__ W) {
-  extern __shared__ float cs_raw[];
+  extern __shared__ __align__(16) float cs_raw[];
   const int nt = (b + kCT - 1) / kCT;
   const int ntiles = nt * (nt + 1) / 2;
-  float* Ts = cs_raw;                                   // [ntiles][32][33]
-  float* Ss = Ts + (size_t)ntiles * kCT * kCLd;         // [nt - 1][32][33] scratch
+  float* Ts = cs_raw;                                   // [ntiles][32][kCLd]
+  float* Ss = Ts + (size_t)ntiles * kCT * kCLd;         // [nt - 1][32][kCLd] scratch
   float* gd = Ss + (size_t)(nt > 1 ? nt - 1 : 1) * kCT * kCLd;  // [32 nt]
   int* sdrop = reinterpret_cast<int*>(gd + kCT * nt);   // [32 nt]
+  __shared__ __align__(16) float cbuf[2][kCT];          // a column of the diagonal tile, by parity
+  __shared__ __align__(16) float Dt[kCT][kCT];          // the diagonal tile by columns
+  __shared__ float dinv[kCT];                           // 1 / pivot (0: dropped)
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = kChThreads / 32;
   auto T = [&](int I, int J) { return Ts + (size_t)ctile(I, J) * kCT * kCLd; };
-  // symmetrised copy, thread = (r, c) of every tile (kCT x kCT / kChThreads
-  // passes); rows/columns beyond b padded with the identity
-  for (int rc = tid; rc < kCT * kCT; rc += kChThreads) {
-    const int r = rc % kCT, c = rc / kCT;
-    int I = 0, J = 0;
-#pragma unroll 4
-    for (int t = 0; t < ntiles; ++t) {
-      const int gi = I * kCT + r, gj = J * kCT + c;
-      float v;
-      if (gi < b && gj < b) v = (float)(0.5 * (G[gi + (size_t)gj * ldg] + G[gj + (size_t)gi * ldg]));
-      else v = (gi == gj) ? 1.f : 0.f;
-      Ts[(size_t)t * kCT * kCLd + r * kCLd + c] = v;
-      if (++J > I) {
-        ++I;
-        J = 0;
-      }
+  // symmetrised copy, a warp per 8 columns of a tile; rows/columns beyond b
+  // padded with the identity.  An entry equal to its mirror (a Gram matrix as
+  // this library forms it) needs no FP64 sum.
+  for (int t = warp; t < 4 * ntiles; t += nw) {
+    int I = 0;
+    while ((I + 1) * (I + 2) / 2 <= (t >> 2)) ++I;
+    const int J = (t >> 2) - I * (I + 1) / 2, c0 = (t & 3) * 8, gi = I * kCT + lane;
+    float* D = T(I, J) + lane * kCLd;
+    double x[8], y[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int gj = J * kCT + c0 + u;
+      const bool in = gi < b && gj < b;
+      x[u] = in ? G[gi + (size_t)gj * ldg] : (gi == gj ? 1.0 : 0.0);
+      y[u] = in ? G[gj + (size_t)gi * ldg] : (gi == gj ? 1.0 : 0.0);
+    }
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const bool same = __double_as_longlong(x[u]) == __double_as_longlong(y[u]);
+      if (!__all_sync(0xffffffffu, same)) x[u] = 0.5 * (x[u] + y[u]);
+      D[c0 + u] = (float)x[u];
     }
   }
   for (int i = tid; i < kCT * nt; i += kChThreads) gd[i] = i < b ? (float)G[i + (size_t)i * ldg] : 1.f;
@@ -611,31 +647,48 @@ __global__ void __launch_bounds__(kChThreads, 1) k_chol_inv_blocked(int b, const
     float* D = T(k, k);
     if (warp == 0) {
       // lane r holds the trailing part of row r (columns j..31 in a[0..31-j],
-      // shifted left after every column, so the current column is a[0] and
-      // the loop over j stays rolled); column j travels by shuffle
+      // shifted left with every column, so the current column is a[0] and the
+      // loop over j stays rolled); the part of a row above the diagonal is
+      // carried along and never used
       float a[kCT];
 #pragma unroll
-      for (int c = 0; c < kCT; ++c) a[c] = D[lane * kCLd + c];
+      for (int c = 0; c < kCT; c += 4) {
+        const float4 v = *reinterpret_cast<const float4*>(D + lane * kCLd + c);
+        a[c] = v.x;
+        a[c + 1] = v.y;
+        a[c + 2] = v.z;
+        a[c + 3] = v.w;
+      }
       for (int j = 0; j < kCT; ++j) {
         const float d = __shfl_sync(0xffffffffu, a[0], j);
         const float g0 = gd[k * kCT + j];
         const bool keep = g0 > 0.f && d > 64.f * 0x1p-24f * g0;
-        const float ljj = keep ? sqrtf(d) : 1.f;
-        if (lane > j) a[0] = keep ? a[0] / ljj : 0.f;
-        if (lane == j) {
-          a[0] = ljj;
-          if (!keep)
-            for (int c = 0; c < j; ++c) D[j * kCLd + c] = 0.f;
+        // 1 / sqrt(d) with a Newton step, sqrt(d) = d / sqrt(d)
+        float inv = rsqrtf(d);
+        inv = inv * fmaf(-0.5f * d * inv, inv, 1.5f);
+        if (!keep) inv = 0.f;
+        const float l = lane > j ? (keep ? a[0] * inv : 0.f) : lane == j ? (keep ? d * inv : 1.f) : 0.f;
+        cbuf[j & 1][(lane - j) & 31] = l;  // entry u: row j + u (rows < j: zeros behind)
+        Dt[j][lane] = l;
+        if (lane >= j) D[lane * kCLd + j] = l;  // column j of L (and the diagonal)
+        if (!keep && lane < j) D[j * kCLd + lane] = 0.f;
+        if (lane == 0) {
+          dinv[j] = inv;
+          sdrop[k * kCT + j] = keep ? 0 : 1;
         }
-        if (lane == 0) sdrop[k * kCT + j] = keep ? 0 : 1;
-        if (lane >= j) D[lane * kCLd + j] = a[0];  // column j of L (and the diagonal)
+        __syncwarp();
+        float cv[kCT];
 #pragma unroll
-        for (int u = 1; u < kCT; ++u) {
-          const float lcj = __shfl_sync(0xffffffffu, a[0], (j + u) & 31);
-          if (keep && j + u < kCT && lane >= j + u) a[u] = fmaf(-a[0], lcj, a[u]);
+        for (int u = 0; u < kCT; u += 4) {
+          const float4 v = *reinterpret_cast<const float4*>(&cbuf[j & 1][u]);
+          cv[u] = v.x;
+          cv[u + 1] = v.y;
+          cv[u + 2] = v.z;
+          cv[u + 3] = v.w;
         }
+        const float nl = lane > j ? -l : 0.f;
 #pragma unroll
-        for (int u = 0; u < kCT - 1; ++u) a[u] = a[u + 1];
+        for (int u = 1; u < kCT; ++u) a[u - 1] = fmaf(nl, cv[u], a[u]);
       }
     }
     __syncthreads();
@@ -644,20 +697,38 @@ __global__ void __launch_bounds__(kChThreads, 1) k_chol_inv_blocked(int b, const
       const int J = e / (kCT * kCT), rc = e % (kCT * kCT), r = rc / kCT, c = rc % kCT;
       if (sdrop[k * kCT + r]) T(k, J)[r * kCLd + c] = 0.f;
     }
-    // panel tiles below: row x of tile (I, k) solves x L(k,k)^T = a
+    // panel tiles below: row x of tile (I, k) solves x L(k,k)^T = a (a dropped
+    // row of L(k,k) is zero left of its diagonal, Dt's columns still hold it:
+    // its x is zero all the same)
     for (int row = tid; row < (nt - 1 - k) * kCT; row += kChThreads) {
       const int I = k + 1 + row / kCT, r = row % kCT;
       float* a = T(I, k) + r * kCLd;
       float x[kCT];
 #pragma unroll
-      for (int j = 0; j < kCT; ++j) {
-        float v = a[j];
-#pragma unroll
-        for (int l = 0; l < j; ++l) v = fmaf(-x[l], D[j * kCLd + l], v);
-        x[j] = sdrop[k * kCT + j] ? 0.f : v / D[j * kCLd + j];
+      for (int j = 0; j < kCT; j += 4) {
+        const float4 v = *reinterpret_cast<const float4*>(a + j);
+        x[j] = v.x;
+        x[j + 1] = v.y;
+        x[j + 2] = v.z;
+        x[j + 3] = v.w;
       }
 #pragma unroll
-      for (int j = 0; j < kCT; ++j) a[j] = x[j];
+      for (int l = 0; l < kCT; ++l) {
+        const float di = dinv[l];
+        x[l] = di != 0.f ? x[l] * di : 0.f;
+        const float nx = -x[l];
+        asm volatile("" ::: "memory");  // the next column's reads stay behind: they would not fit the registers
+#pragma unroll
+        for (int j = (l + 1) & ~3; j < kCT; j += 4) {
+          const float4 v = *reinterpret_cast<const float4*>(&Dt[l][j]);
+          if (j > l) x[j] = fmaf(nx, v.x, x[j]);
+          if (j + 1 > l) x[j + 1] = fmaf(nx, v.y, x[j + 1]);
+          if (j + 2 > l) x[j + 2] = fmaf(nx, v.z, x[j + 2]);
+          if (j + 3 > l) x[j + 3] = fmaf(nx, v.w, x[j + 3]);
+        }
+      }
+#pragma unroll
+      for (int j = 0; j < kCT; j += 4) *reinterpret_cast<float4*>(a + j) = make_float4(x[j], x[j + 1], x[j + 2], x[j + 3]);
     }
     __syncthreads();
     // trailing update A(I,J) -= L(I,k) L(J,k)^T, k < J <= I
@@ -667,7 +738,7 @@ __global__ void __launch_bounds__(kChThreads, 1) k_chol_inv_blocked(int b, const
         int I = 0;
         while ((I + 1) * (I + 2) / 2 <= t) ++I;
         const int J = t - I * (I + 1) / 2;
-        warp_tile_mac(T(k + 1 + I, k + 1 + J), T(k + 1 + I, k), T(k + 1 + J, k), true, -1.f, lane);
+        warp_tile_sub(T(k + 1 + I, k + 1 + J), T(k + 1 + I, k), T(k + 1 + J, k), lane);
       }
     }
     __syncthreads();
@@ -702,10 +773,7 @@ __global__ void __launch_bounds__(kChThreads, 1) k_chol_inv_blocked(int b, const
 #pragma unroll
         for (int l = 0; l < kCT; ++l) bv[l] = B[l * kCLd + lane];
 #pragma unroll
-        for (int rr = 0; rr < 8; ++rr) {
-#pragma unroll
-          for (int l = 0; l < kCT; ++l) acc[rr] = fmaf(A[(r0 + rr) * kCLd + l], bv[l], acc[rr]);
-        }
+        for (int rr = 0; rr < 8; ++rr) acc[rr] = tile_row_dot(A + (r0 + rr) * kCLd, bv, acc[rr]);
       }
 #pragma unroll
       for (int rr = 0; rr < 8; ++rr) S[(r0 + rr) * kCLd + lane] = acc[rr];
@@ -720,22 +788,16 @@ __global__ void __launch_bounds__(kChThreads, 1) k_chol_inv_blocked(int b, const
       for (int l = 0; l < kCT; ++l) bv[l] = B[l * kCLd + lane];
       float* X = T(I, K);
 #pragma unroll
-      for (int rr = 0; rr < 8; ++rr) {
-        float acc = 0.f;
-#pragma unroll
-        for (int l = 0; l < kCT; ++l) acc = fmaf(A[(r0 + rr) * kCLd + l], bv[l], acc);
-        X[(r0 + rr) * kCLd + lane] = -acc;
-      }
+      for (int rr = 0; rr < 8; ++rr) X[(r0 + rr) * kCLd + lane] = -tile_row_dot(A + (r0 + rr) * kCLd, bv, 0.f);
     }
     __syncthreads();
   }
   for (int i = tid; i < b; i += kChThreads) dropped[i] = sdrop[i];
-  // W0 = (L^-1)^T, dropped columns zero
-  for (int e = tid; e < b * b; e += kChThreads) {
-    const int i = e % b, j = e / b;
-    float v = 0.f;
-    if (!sdrop[j] && j >= i) v = T(j / kCT, i / kCT)[(j % kCT) * kCLd + (i % kCT)];
-    W[i + (size_t)j * b] = (double)v;
+  // W0 = (L^-1)^T, dropped columns zero; a warp per column of W
+  for (int j = warp; j < b; j += nw) {
+    const bool dj = sdrop[j] != 0;
+    for (int i = lane; i < b; i += 32)
+      W[i + (size_t)j * b] = !dj && j >= i ? widen(T(j / kCT, i / kCT)[(j % kCT) * kCLd + (i % kCT)]) : 0.0;
   }
 }
 
