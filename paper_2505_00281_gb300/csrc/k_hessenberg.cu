@@ -1222,6 +1222,11 @@ __global__ void __launch_bounds__(kRowThreads + 32 * kMaxPoll, 1) k_hess_row(
   __shared__ unsigned long long s_key[2][kRowThreads / 32];
   __shared__ float s_l[kPw][kPw];
   __shared__ int s_kept[kPw], s_bad[3];
+  if constexpr (CL)
+    if (cooperative_groups::this_cluster().num_blocks() != gridDim.x) {
+      if (tid == 0) atomicCAS(ws.err, 0, (int)RR_ERR_CUDA);
+      return;  // every CTA alike
+    }
 
   for (int c = warp; c < k; c += nwarps) {
     const float* src = W + r0 + (int64_t)c * ldw;
@@ -1567,7 +1572,11 @@ static rr_status hess_res_launch(int64_t n, int64_t k, float* W, int64_t ldw, TO
   int rt = byrow ? (p.rpc + 31) / 32 * 32 : kRowThreads;
   const unsigned threads = rt + 32 * ((p.G + 31) / 32);
   // one cluster where the CTAs fit one (checked against the GPU's cluster
-  // occupancy): the words go through distributed shared memory
+  // occupancy): the words go through distributed shared memory, and the
+  // cluster's own co-scheduling stands in for a cooperative launch (the two
+  // attributes together are not kept by every tool that replays a launch, and
+  // without its cluster the kernel would address memory that is not there: it
+  // checks)
   const void* fn = (const void*)k_hess_row<TO, true>;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(p.G);
@@ -1581,8 +1590,8 @@ static rr_status hess_res_launch(int64_t n, int64_t k, float* W, int64_t ldw, TO
   at[1].val.clusterDim.x = p.G;
   at[1].val.clusterDim.y = 1;
   at[1].val.clusterDim.z = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 2;
+  cfg.attrs = at + 1;
+  cfg.numAttrs = 1;
   bool cl = false;
   if (byrow && p.G <= kHessMaxCluster) {
     RR_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
@@ -1593,7 +1602,7 @@ static rr_status hess_res_launch(int64_t n, int64_t k, float* W, int64_t ldw, TO
   }
   if (!cl) {
     fn = byrow ? (const void*)k_hess_row<TO, false> : (const void*)k_hess_res<TO>;
-    cfg.numAttrs = 1;
+    cfg.attrs = at;
     RR_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   }
   Arena ar(mem, hess_res_bytes(kmem));
