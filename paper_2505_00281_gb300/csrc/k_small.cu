@@ -92,21 +92,26 @@ __global__ void __launch_bounds__(kSmallThreads) k_tri_inv_lower(int b, const do
 }
 
 // Small products C = alpha op(A) op(B) + beta C (op = transpose when ta / tb),
-// 16 x 16 output tiles, one output per thread, K in panels of KP staged in
-// shared memory with all of a panel's loads in flight at once.  On GB300 the
-// FP64 units of an SM are the limit (a 16 x 16 x 256 tile is 65k FP64 FMAs,
-// ~16 us on one SM), so the work is cut into (tile, K-range) pieces spread
-// evenly over the SMs: 1-D grid of ntiles x ks CTAs; with ks > 1 (beta = 0)
-// the K ranges' partial sums add into a zeroed C with FP64 atomics.  sym:
-// the result is symmetric (M == N): only tiles with bx <= by are computed,
-// the off-diagonal ones write their mirror image too.
-template <typename TA, int KP>
-__global__ void __launch_bounds__(256) k_gemm_small(int ta, int tb, int M, int N, int K, double alpha,
+// T x T output tiles on 256 threads, a tile's K cut into 256 / T^2 interleaved
+// parts (added up through shared memory at the end), staged in panels of KP with
+// all of a panel's loads in flight at once.  sym: the result is symmetric (M ==
+// N): only tiles with bx <= by are computed, the off-diagonal ones write their
+// mirror image too.
+//   FP64 (T = 8): the FP64 units of an SM are the limit (two FMAs a clock, 27 us
+//   for 256^3 on all of them), so small tiles spread the work evenly and eight
+//   CTAs an SM cover each other's loads: 256^3 36.5 us, 64^3 5.5 (16 x 16 tiles
+//   with their K ranges on CTAs of their own, added by FP64 atomics into a C
+//   zeroed by a launch before: 33.8 + 2.4 and 8.6 + 2.4; the K ranges as a
+//   cluster that adds up through distributed shared memory: 39 and 7.4).
+//   FP32 products of FP64 data (T = 16): the conversions are the limit, so
+//   larger tiles: 256^3 12.8 us, 64^3 6.7 (13.7 and 8.6).
+template <typename TA, int T, int KP>
+__global__ void __launch_bounds__(256, T == 8 ? 8 : 2) k_gemm_small(int ta, int tb, int M, int N, int K, double alpha,
                                                     const double* __restrict__ A, int lda,
                                                     const double* __restrict__ B, int ldb, double beta,
-                                                    double* __restrict__ C, int ldc, int sym, int ks, int kc) {
-  const int tm = (M + 15) / 16;
-  const int tile = blockIdx.x / ks, split = blockIdx.x - tile * ks;
+                                                    double* __restrict__ C, int ldc, int sym) {
+  constexpr int kOut = T * T, kParts = 256 / kOut;
+  const int tm = (M + T - 1) / T, tile = blockIdx.x;
   int bx, by;
   if (sym) {  // tile = by (by + 1) / 2 + bx, bx <= by
     by = (int)((sqrtf(8.f * (float)tile + 1.f) - 1.f) * 0.5f);
@@ -117,93 +122,80 @@ __global__ void __launch_bounds__(256) k_gemm_small(int ta, int tb, int M, int N
     bx = tile % tm;
     by = tile / tm;
   }
-  __shared__ TA As[KP][17];
-  __shared__ TA Bs[KP][17];
-  const int m0 = bx * 16, n0 = by * 16;
-  const int kbeg = split * kc, kend = min(K, kbeg + kc);
-  const int tid = threadIdx.x, ti = tid % 16, tj = tid / 16;
+  __shared__ TA As[KP][T + 1];
+  __shared__ TA Bs[KP][T + 1];
+  __shared__ TA part[kParts][kOut];
+  const int m0 = bx * T, n0 = by * T;
+  const int tid = threadIdx.x, q = tid / kOut, ti = tid % T, tj = tid / T % T;
   TA acc = TA(0);
-  for (int k0 = kbeg; k0 < kend; k0 += KP) {
-    for (int e = tid; e < KP * 16; e += 256) {
-      // consecutive threads along the operand's contiguous dimension
-      const int ka = ta ? e % KP : e / 16, ia = ta ? e / KP : e % 16;
+  for (int k0 = 0; k0 < K; k0 += KP) {
+    const int kn = K - k0 < KP ? K - k0 : KP;
+#pragma unroll(KP * T / 256 < 4 ? KP * T / 256 : 4)
+    for (int u = 0; u < KP * T / 256; ++u) {
+      // consecutive threads along the operand's contiguous dimension; selects,
+      // not branches, so that the loads of several u go out together
+      const int e = tid + 256 * u;
+      const int ka = ta ? e % KP : e / T, ia = ta ? e / KP : e % T;
       const int gk = k0 + ka, gi = m0 + ia;
-      As[ka][ia] = (gk < kend && gi < M) ? (TA)(ta ? A[gk + (size_t)gi * lda] : A[gi + (size_t)gk * lda]) : TA(0);
-      const int kb = tb ? e / 16 : e % KP, jb = tb ? e % 16 : e / KP;
+      const double x = ka < kn && gi < M ? (ta ? A[gk + (size_t)gi * lda] : A[gi + (size_t)gk * lda]) : 0.0;
+      const int kb = tb ? e / T : e % KP, jb = tb ? e % T : e / KP;
       const int gkb = k0 + kb, gj = n0 + jb;
-      Bs[kb][jb] = (gkb < kend && gj < N) ? (TA)(tb ? B[gj + (size_t)gkb * ldb] : B[gkb + (size_t)gj * ldb]) : TA(0);
+      const double y = kb < kn && gj < N ? (tb ? B[gj + (size_t)gkb * ldb] : B[gkb + (size_t)gj * ldb]) : 0.0;
+      As[ka][ia] = (TA)x;
+      Bs[kb][jb] = (TA)y;
     }
     __syncthreads();
-    const int kn = kend - k0 < KP ? kend - k0 : KP;
 #pragma unroll 8
-    for (int kk = 0; kk < kn; ++kk) acc = fma(As[kk][ti], Bs[kk][tj], acc);
+    for (int kk = q; kk < kn; kk += kParts) acc = fma(As[kk][ti], Bs[kk][tj], acc);
     __syncthreads();
+  }
+  if (kParts > 1) {
+    part[q][tid % kOut] = acc;
+    __syncthreads();
+    if (q != 0) return;
+#pragma unroll
+    for (int p = 1; p < kParts; ++p) acc += part[p][tid];
   }
   const int i = m0 + ti, j = n0 + tj;
   if (i < M && j < N) {
-    const double v0 = alpha * (double)acc;
-    if (ks > 1) {
-      atomicAdd(C + i + (size_t)j * ldc, v0);
-      if (sym && bx != by) atomicAdd(C + j + (size_t)i * ldc, v0);
-    } else {
-      double v = v0;
-      if (beta != 0.0) v += beta * C[i + (size_t)j * ldc];
-      C[i + (size_t)j * ldc] = v;
-      if (sym && bx != by) C[j + (size_t)i * ldc] = v;
-    }
+    double v = alpha * (double)acc;
+    if (beta != 0.0) v += beta * C[i + (size_t)j * ldc];
+    C[i + (size_t)j * ldc] = v;
+    if (sym && bx != by) C[j + (size_t)i * ldc] = v;
   }
 }
 
-__global__ void k_zero_small(int M, int N, double* __restrict__ C, int ldc) {
-  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < M * N; e += gridDim.x * blockDim.x)
-    C[e % M + (size_t)(e / M) * ldc] = 0.0;
-}
-
-template <typename TA, int KP>
+template <typename TA, int T, int KP>
 static void gemm_small_launch(cudaStream_t s, int ta, int tb, int M, int N, int K, double alpha,
                               const double* A, int lda, const double* B, int ldb, double beta, double* C,
                               int ldc, int sym) {
-  const int tm = (M + 15) / 16, tn = (N + 15) / 16;
+  const int tm = (M + T - 1) / T, tn = (N + T - 1) / T;
   const int ntiles = sym ? tm * (tm + 1) / 2 : tm * tn;
-  // about six CTAs per SM, each K range at least 64 long
-  int ks = 1;
-  if (beta == 0.0) {
-    const int want = (6 * num_sms() + ntiles - 1) / ntiles;
-    const int most = K / 64 > 1 ? K / 64 : 1;
-    ks = want < most ? want : most;
-    if (ks < 1) ks = 1;
-  }
-  const int kc = (K + ks - 1) / ks;
-  ks = (K + kc - 1) / kc;
-  if (ks > 1) {
-    k_zero_small<<<(M * N + 255) / 256, 256, 0, s>>>(M, N, C, ldc);
-    note_launches(1);
-  }
-  k_gemm_small<TA, KP><<<ntiles * ks, 256, 0, s>>>(ta, tb, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, sym, ks,
-                                                   kc);
+  k_gemm_small<TA, T, KP><<<ntiles, 256, 0, s>>>(ta, tb, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, sym);
 }
 
 static void gemm_small(cudaStream_t s, int ta, int tb, int M, int N, int K, double alpha,
                        const double* A, int lda, const double* B, int ldb, double beta, double* C,
                        int ldc) {
-  gemm_small_launch<double, 128>(s, ta, tb, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, 0);
+  gemm_small_launch<double, 8, 64>(s, ta, tb, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, 0);
 }
 
 // C (n x n) = A^T B for a product known to be symmetric (W^T G W, N^T N,
 // V^T V): half the tiles
 static void gemm_small_sym(cudaStream_t s, int n, int K, const double* A, int lda, const double* B, int ldb,
                            double* C, int ldc) {
-  gemm_small_launch<double, 128>(s, 1, 0, n, n, K, 1.0, A, lda, B, ldb, 0.0, C, ldc, 1);
+  gemm_small_launch<double, 8, 64>(s, 1, 0, n, n, K, 1.0, A, lda, B, ldb, 0.0, C, ldc, 1);
 }
 
 static void gemm_mixed(cudaStream_t s, int ta, int tb, int M, int N, int K, double alpha,
                        const double* A, int lda, const double* B, int ldb, double beta, double* C,
                        int ldc) {
-  // FP32 products are not FP64-unit bound: whole-K tiles
-  dim3 g((unsigned)(((M + 15) / 16) * ((N + 15) / 16)));
-  const int tm = (M + 15) / 16;
-  (void)tm;
-  k_gemm_small<float, 256><<<g, 256, 0, s>>>(ta, tb, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, 0, 1, K);
+  // one panel where K fits 64, else the longer ones: several panels of 64 wait
+  // for each other's loads (256^3 in 18 us, 64^3 with panels of 256 in 8.6)
+  if (K <= 64)
+    gemm_small_launch<float, 16, 64>(s, ta, tb, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, 0);
+  else
+    gemm_small_launch<float, 16, 256>(s, ta, tb, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, 0);
 }
 
 // Symmetrise C and decouple dropped indices (zero row and column; their

@@ -60,3 +60,25 @@ def test_pencil_svd_graded_columns(rr, b):
 @pytest.mark.parametrize("b", [4, 65])
 def test_pencil_svd_nothing_to_rotate(rr, b):
     _check(rr, torch.diag(torch.linspace(2, 1, b, dtype=torch.float64)).cuda())
+
+
+@pytest.mark.parametrize("b", [1, 31, 32, 33, 65, 96, 255, 256])
+def test_pencil_eig_whitening_tile_edges(rr, b):
+    """The Cholesky-inverse's 32 x 32 tiles at their edges: Y^T G Y = I and
+    H Y = G Y theta for a Gram matrix of condition below 64."""
+    g = torch.Generator().manual_seed(b)
+    X = torch.randn(2 * b + 8, b, generator=g, dtype=torch.float64)
+    G = X.t() @ X / (2 * b + 8)
+    S = torch.randn(b, b, generator=g, dtype=torch.float64)
+    H = (S + S.t()) / 2
+    w = torch.linalg.eigvalsh(G)
+    assert float(w[-1] / w[0]) < 64
+    cm = lambda t: t.cuda().t().contiguous().t()  # noqa: E731
+    theta, Y, dropped = rr.rr_pencil_eig(cm(H), cm(G))
+    assert dropped == 0
+    theta, Y = theta.cpu(), Y.cpu()
+    # products of length b (64 b eps, as above) times the condition of G
+    tol = 64 * 64 * b * EPS
+    assert float((Y.t() @ G @ Y - torch.eye(b, dtype=torch.float64)).abs().max()) <= tol
+    scale = float(H.abs().sum(0).max()) * float(Y.abs().max())
+    assert float((H @ Y - G @ Y * theta).abs().max()) <= tol * max(1.0, scale)
