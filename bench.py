@@ -191,12 +191,12 @@ def aggregate(seconds: float, converged: int, dist=None, device=None):
 
 
 # --------------------------------------------------------------------------- GPU arm
-# DRAM bytes per launch of k_gemm_bf16_tc by role (the low-precision products,
-# the FP64-emulation passes), mean over one solve of this workload (ncu
+# DRAM bytes per launch by role (the low-precision products of k_gemm_bf16_tc;
+# the FP64-emulation passes of k_emu_mm), mean over one solve of this workload (ncu
 # dram__bytes_read.sum + dram__bytes_write.sum, a one-pass capture of every
 # launch of the kernel in one solve; profiles/ncu_gemm_bf16_tc_16384x4096x128.md).
 # Emptied when the kernel changes, until it is captured again.
-TC_TRAFFIC_PER_LAUNCH = {"lowp_product": 221.6e6, "f64_emulation": 231.7e6}
+TC_TRAFFIC_PER_LAUNCH = {"lowp_product": 221.6e6}
 
 
 def stage_roofline(info, peaks, src):
@@ -204,16 +204,14 @@ def stage_roofline(info, peaks, src):
     stage of one solve) with each stage's share, and the roofline of the
     dominant kernel.
 
-    ``roofline`` is the tcgen05 product kernel ``k_gemm_bf16_tc``, the
-    dominant kernel, whose launches play two roles: the low-precision
-    products (filter products, split-BF16 corrections; HBM-bound at b = 128,
-    128 flop per byte of operator against a BF16 ridge near 260) and the
-    FP64-emulation passes (all slice pairs of an FP64-accurate product, Gram
-    or lift in one launch: 36 pair products per operator slice set, above the
-    ridge, so tensor-bound).  The library brackets every launch with CUDA
+    ``roofline`` is the tcgen05 product work in two roles: the low-precision
+    products of ``k_gemm_bf16_tc`` (filter products, split-BF16 corrections;
+    HBM-bound at b = 128, 128 flop per byte of operator against a BF16 ridge
+    near 260) and the FP64-emulation passes of ``k_emu_mm`` (all slice pairs of
+    an FP64-accurate product, Gram or lift in one launch: 28 pair products of
+    slices formed on chip, above the ridge, so tensor-bound).  The library brackets every launch with CUDA
     events on its stream and adds up, per role, its algorithmic bytes (each
-    operand read once -- for an emulation pass the distinct 6-bit slices --
-    and the output written once) and flops (2 M N K per product formed).  The
+    operand read once, the output written once) and flops (2 M N K per product formed).  The
     line carries the role that holds most of the kernel's time against its
     own bound; ``roles`` gives both, and ``kernel_roofline_time_frac`` the
     roofline time of every launch (max of bytes / measured bandwidth and
@@ -283,7 +281,7 @@ def stage_roofline(info, peaks, src):
                     "frac": d["achieved_gbs"] / hbm}
         roof.update({"traffic": TC_TRAFFIC_PER_LAUNCH.get(main),
                      "traffic_scope": "DRAM bytes per launch of this role (mean over one solve, ncu)",
-                     "kernel": "k_gemm_bf16_tc", "role": main, "launches": tc_n,
+                     "kernel": {"lowp_product": "k_gemm_bf16_tc", "f64_emulation": "k_emu_mm"}[main], "role": main, "launches": tc_n,
                      "kernel_ms_per_solve": tc_ms, "kernel_share_of_solve": tc_ms / total if total else None,
                      "role_share_of_kernel": d["ms"] / tc_ms, "roles": roles,
                      "kernel_roofline_time_frac": t_roof / tc_ms,

@@ -288,11 +288,11 @@ rr_status rr_split_operator(int64_t m, int64_t n, const double* A, int64_t lda, 
  *   X (n x b, ld ldx) = S1 (n x p1, ld ld1) Y(0:p1, :) + S2 (n x p2, ld ld2) Y(p1:p1+p2, :)
  * with Y FP64 (p1+p2) x b (ld ldy), all column-major; S1, S2 of type t1, t2
  * (RR_F64, RR_F32 or RR_BF16); S2 may be NULL (p2 ignored).  FP64-accurate:
- * when p1+p2 is a multiple of 8 and at most 512, b <= 256 and ws holds
+ * when p1+p2 is at most 512, b <= 256 and ws holds
  * rr_lift_workspace_size(n, b, p1+p2) bytes, the product runs on the BF16
- * tensor cores through error-free 6-bit slices of both operands (per-entry
- * error below (p1+p2) 2^-47 max_k|S(i,k)| max_k|Y(k,j)|); otherwise in FP64
- * arithmetic.  RR_ERR_ARG: negative sizes, p1 < 1, b < 1, bad type or NULL
+ * tensor cores through error-free 7-bit slices of both operands, formed on
+ * chip (per-entry error below (p1+p2) 2^-47 max_k|S(i,k)| max_k|Y(k,j)|, each
+ * block of S with its own row maxima); otherwise in FP64 arithmetic.  RR_ERR_ARG: negative sizes, p1 < 1, b < 1, bad type or NULL
  * pointers. */
 size_t rr_lift_workspace_size(int64_t n, int64_t b, int64_t K);
 rr_status rr_lift(int64_t n, int64_t b, int32_t t1, const void* S1, int64_t ld1, int64_t p1,
@@ -333,13 +333,13 @@ rr_status rr_gemm_f64(int32_t trans, int64_t M, int64_t N, int64_t K, const doub
 /* FP64-accurate product C = op(A) B on the BF16 tensor cores (error-free
  * fixed-point slicing): op(A) as in rr_gemm_f64, A and B FP64, C FP64.
  * Rows of A (trans = 0) or columns of A (trans = 1) and columns of B are
- * scaled by powers of two and split into `slices` (1..10) integer BF16
- * slices of 6 bits; every slice product is exact in the FP32 tensor-core
- * accumulator (K-chunks of at most 4096), and is scaled and summed in FP64.
- * With 8 slices the result agrees with FP64 arithmetic to about 2^-54 of
- * |op(A)| |B|.  N <= 256; the row strides of op(A)'s K-major copy (m and n)
- * must be multiples of 8.  Needs rr_gemm_f64_emulated_workspace_size bytes
- * (it holds the slices of A and B). */
+ * scaled by powers of two and cut on chip into integer BF16 slices of 7 bits
+ * (7 of them for `slices` 1..8, 9 for 9 and 10); the pair products are exact
+ * in the FP32 tensor-core accumulator (448 columns of K at a time) and are
+ * combined in 64-bit integers.  With 7 slices the result agrees with FP64
+ * arithmetic to about 2^-54 of |op(A)| |B|.  N <= 256; m and n must be
+ * multiples of 8.  Needs rr_gemm_f64_emulated_workspace_size bytes (exponents
+ * and the slices of B). */
 size_t rr_gemm_f64_emulated_workspace_size(int32_t trans, int64_t M, int64_t N, int64_t K,
                                            int32_t slices);
 rr_status rr_gemm_f64_emulated(int32_t trans, int64_t M, int64_t N, int64_t K, const double* A,
@@ -356,7 +356,10 @@ rr_status rr_gemm_f64_emulated(int32_t trans, int64_t M, int64_t N, int64_t K, c
  * smallest row index.  Arithmetic is IEEE with separately rounded multiply
  * and subtract (no FMA contraction), so results are reproducible bit for bit.
  * Needs rr_hessenberg_workspace_size(n, k, arith) bytes of workspace.
- * Runs as one cooperative launch with one grid barrier per column. */
+ * FP32: one launch where the block fits the CTAs' shared memory (one cluster
+ * up to 16 CTAs, a cooperative grid above, panels of 8 columns, one exchange
+ * per column), panels of 32 columns otherwise; FP64: one cooperative launch
+ * with one grid barrier per column. */
 size_t rr_hessenberg_workspace_size(int64_t n, int64_t k, int32_t arith);
 rr_status rr_hessenberg(int32_t arith, int64_t n, int64_t k, void* W, int64_t ldw,
                         int32_t qtype, void* Q, int64_t ldq, int32_t* piv, double tol,
@@ -372,7 +375,7 @@ rr_status rr_hessenberg(int32_t arith, int64_t n, int64_t k, void* W, int64_t ld
  * T -= L_panel W.  Every entry sees the same separately rounded operations in
  * the same order as in rr_hessenberg, so W, Q and piv equal its results bit
  * for bit; the trailing columns are streamed once per panel instead of once
- * per column.  rr_hessenberg takes this path by itself (panel 16) when a
+ * per column.  rr_hessenberg takes this path by itself (panel 32) when a
  * CTA's share of rows of all k columns does not fit its shared memory.
  * W: n x k FP32 (ld ldw, overwritten); Q: qtype RR_F32, RR_BF16 or RR_F64;
  * n < 2^24.  Workspace: rr_hessenberg_workspace_size(n, k, RR_F32).
@@ -436,12 +439,11 @@ rr_status rr_basis_builder(int32_t method, int32_t storage, int64_t n, int64_t k
 /* Projection products (Alg. 3: B = U^T A U, M = U^T U; Alg. 5: U^T A V,
  * U^T U, V^T V): G (p x q FP64, ld ldg) = X^T Y (+ G if accumulate) for tall
  * X (n x p) and Y (n x q) of types xtype/ytype (RR_F64, RR_F32, RR_BF16).
- * FP64-accurate: when n >= 64 and n % 8 == 0 the products run on the tensor
- * cores (in column chunks of at most 128 of Y) from 8 column-scaled 6-bit
- * slices of each operand with
- * exact FP32 sums over 4096-long K chunks (error per entry below
+ * FP64-accurate: when n >= 64 the products run on the tensor cores from 7
+ * column-scaled 7-bit slices of each operand, formed on chip, with exact FP32
+ * sums over 448 rows at a time (error per entry below
  * 2^-47 n max|X(:,i)| max|Y(:,j)|); otherwise FP64 accumulation on the CUDA
- * cores.  Needs rr_gram_workspace_size(n, p, q) bytes (slices and
+ * cores.  Needs rr_gram_workspace_size(n, p, q) bytes (exponents and
  * deterministic split-K partials, reduced in a fixed order). */
 size_t rr_gram_workspace_size(int64_t n, int64_t p, int64_t q);
 rr_status rr_gram(int64_t n, int64_t p, int64_t q, int32_t xtype, const void* X, int64_t ldx,
