@@ -861,8 +861,8 @@ __global__ void __launch_bounds__(256) k_emu_bslice(int64_t K, int64_t N, const 
 }
 
 // Exponents of the largest entry of every column (atomic maxima over row
-// chunks, so that a tall block's few columns fill the GPU; e starts very
-// negative).  8 loads in flight a thread; bound by HBM.
+// chunks, so that a tall block's few columns fill the GPU; e then starts very
+// negative; a plain store with one chunk).  8 loads in flight a thread; bound by HBM.
 template <typename TS>
 __global__ void __launch_bounds__(256) k_emu_col_exp(int64_t n, const TS* __restrict__ X, int64_t ldx, int64_t rpc,
                                                      int* __restrict__ e) {
@@ -877,7 +877,18 @@ __global__ void __launch_bounds__(256) k_emu_col_exp(int64_t n, const TS* __rest
     for (int u = 0; u < 8; ++u) mx = max(mx, exp_raw<TS>(v[u]));
   }
   mx = __reduce_max_sync(0xffffffffu, mx);
-  if ((threadIdx.x & 31) == 0) atomicMax(e + j, mx);
+  if (gridDim.x > 1) {
+    if ((threadIdx.x & 31) == 0) atomicMax(e + j, mx);
+    return;
+  }
+  __shared__ int sm[8];
+  if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = mx;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+#pragma unroll
+    for (int w = 1; w < 8; ++w) mx = max(mx, sm[w]);
+    e[j] = mx;
+  }
 }
 
 // Exponents of the largest entry of every row of a column-major block (lane =
@@ -1032,9 +1043,15 @@ rr_status slice_b(cudaStream_t s, int64_t K, int64_t N, const double* B, int64_t
   return check_launch("emu B slices");
 }
 
+// Row chunks of the column exponents: about 8 blocks an SM over the columns, at
+// least 2048 rows each; one up to 4096 rows, where e then needs no start value
+// (a small Gram is bound by its launches: the memset is one of five).
+int64_t col_exp_chunks(int64_t n, int64_t c) {
+  if (n <= 4096) return 1;
+  return std::max<int64_t>(1, std::min<int64_t>((n + 2047) / 2048, (8 * (int64_t)num_sms() + c - 1) / c));
+}
 rr_status col_exps(cudaStream_t s, int32_t type, int64_t n, int64_t c, const void* X, int64_t ldx, int* e) {
-  // about 8 blocks an SM over the columns, at least 2048 rows each
-  int64_t chunks = std::max<int64_t>(1, std::min<int64_t>((n + 2047) / 2048, (8 * (int64_t)num_sms() + c - 1) / c));
+  int64_t chunks = col_exp_chunks(n, c);
   const int64_t rpc = (n + chunks - 1) / chunks;
   chunks = (n + rpc - 1) / rpc;
   const dim3 g((unsigned)chunks, (unsigned)c);
@@ -1258,7 +1275,8 @@ rr_status emu_gram(cudaStream_t s, int64_t n, int64_t p, int64_t q, int32_t xt, 
   a.part = ar.take<double>((size_t)a.items * 64 * kRows);
   if (ar.overflow) return RR_ERR_WORKSPACE;
   const bool same = X == Y && xt == yt && ldx == ldy && p == q;
-  RR_CUDA(cudaMemsetAsync(ex, 0x80, (size_t)(p + q) * 4, s));  // below every exponent
+  if (col_exp_chunks(n, p) > 1 || (!same && col_exp_chunks(n, q) > 1))
+    RR_CUDA(cudaMemsetAsync(ex, 0x80, (size_t)(p + q) * 4, s));  // below every exponent
   RR_TRY(col_exps(s, xt, n, p, X, ldx, ex));
   if (same) ey = ex;
   else RR_TRY(col_exps(s, yt, n, q, Y, ldy, ey));
