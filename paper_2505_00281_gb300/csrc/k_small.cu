@@ -838,8 +838,8 @@ __global__ void k_whiten_corr(int b, double* __restrict__ E, const double* __res
 // 256 rows takes some 15 thousand clocks (Gram matrix 2.7, 16 sub-rounds of 370
 // clocks, products and exchange 5.1, cluster barrier 2.6) where full-length
 // inner products and column updates in every sub-round took 32 thousand:
-// rr_pencil_svd at 256 x 256 from 5.25 to 4.26 ms, at 320 x 320 (a barrier over
-// the grid instead of the cluster's) from 9.1 to 8.1 ms.
+// this alone took rr_pencil_svd at 256 x 256 from 5.25 to 4.26 ms, at 320 x 320 (a
+// barrier over the grid instead of the cluster's) from 9.1 to 8.1 ms.
 // The rounding of the Gram entries is relative to the two columns' norms, far
 // below the 1e-4 the Jacobi stops at, and the next round starts from fresh
 // ones.  A pair whose inner product is exactly zero, or below tol relative to
@@ -848,7 +848,7 @@ __global__ void k_whiten_corr(int b, double* __restrict__ E, const double* __res
 // padding) stay decoupled.  A round none of whose pairs would rotate skips its
 // sub-rounds; converged when that holds for a whole sweep.
 constexpr int kBJThreads = 512;
-constexpr int kBJMaxChunks = 3;  // float4 row chunks per lane: r, cpad <= 384
+constexpr int kBJMaxRows = 384;  // r, cpad
 
 // (x + y) mod m for 0 <= x, y < m
 __device__ __forceinline__ int add_mod(int x, int y, int m) {
@@ -1783,7 +1783,7 @@ static size_t bj_cl_smem(int r, int cpad, int w) {
 static rr_status launch_bj(cudaStream_t s, int r, int cpad, int w, int P, float* M, float* V, float tol,
                            int max_sweeps, PencilWs& ws, const float* floor_ptr = nullptr) {
   const int rp = (r + 3) & ~3;
-  if (rp > 128 * kBJMaxChunks || cpad > 128 * kBJMaxChunks || 2 * w > 32 || w < 1) return RR_ERR_ARG;
+  if (rp > kBJMaxRows || cpad > kBJMaxRows || 2 * w > 32 || w < 1) return RR_ERR_ARG;
   const size_t csm = bj_cl_smem(r, cpad, w);
   if (P <= kBJMaxCluster && csm <= 220 * 1024) {
     // one cluster: columns stay in shared memory, no global barrier
