@@ -1528,6 +1528,11 @@ __global__ void __launch_bounds__(kRowThreads + 32 * kMaxPoll, 1) k_hess_row(
   }
 }
 
+// Dynamic shared memory a plan may ask for: the 227 KB a CTA can have less 2 KB
+// for the static arrays of the cooperative kernels (1040 bytes, -Xptxas -v).  The
+// cluster form holds 2560 bytes more of them: its launch checks that it fits.
+constexpr int64_t kHessSmem = 225 * 1024;
+
 // rows per CTA, CTAs and the columns that fit in shared memory
 struct HessPlan {
   int G, rpc, kr;
@@ -1537,7 +1542,7 @@ static HessPlan hess_plan(int64_t n, int64_t k) {
   // about 256 rows per CTA (fewer CTAs poll fewer words: 16384 x 128 takes
   // 0.65 ms with 128 rows, 0.50 ms with 256, 0.55 ms with 400), more CTAs where all k columns then fit
   int64_t G = (n + 255) / 256;
-  const int64_t fit = (int64_t)((225 * 1024 - 32 - 36 * k) / (4 * k)) - 1;
+  const int64_t fit = (int64_t)((kHessSmem - 32 - 36 * k) / (4 * k)) - 1;
   if (fit >= 1 && (n + G - 1) / G > fit) G = (n + fit - 1) / fit;
   if (G > num_sms()) G = num_sms();
   if (G > 32 * kMaxPoll) G = 32 * kMaxPoll;
@@ -1546,9 +1551,9 @@ static HessPlan hess_plan(int64_t n, int64_t k) {
   p.G = (int)((n + p.rpc - 1) / p.rpc);
   // a column: its rows, its threshold, its trailing weights
   const size_t per = (size_t)(p.rpc | 1) * 4 + 4 + kPw * 4;
-  p.kr = (int)std::min<int64_t>(k, (int64_t)((225 * 1024 - 32) / per));
+  p.kr = (int)std::min<int64_t>(k, (int64_t)((kHessSmem - 32) / per));
   // the weights are needed only beyond one panel
-  if (p.kr < kPw && p.kr < k) p.kr = (int)std::min<int64_t>(std::min<int64_t>(k, kPw), (int64_t)((225 * 1024 - 32) / ((size_t)(p.rpc | 1) * 4 + 4)));
+  if (p.kr < kPw && p.kr < k) p.kr = (int)std::min<int64_t>(std::min<int64_t>(k, kPw), (int64_t)((kHessSmem - 32) / ((size_t)(p.rpc | 1) * 4 + 4)));
   return p;
 }
 static size_t hess_res_bytes(int64_t k) {
@@ -1576,7 +1581,9 @@ static rr_status hess_res_launch(int64_t n, int64_t k, float* W, int64_t ldw, TO
   // cluster's own co-scheduling stands in for a cooperative launch (the two
   // attributes together are not kept by every tool that replays a launch, and
   // without its cluster the kernel would address memory that is not there: it
-  // checks)
+  // checks).  A slab that leaves no room for the cluster form's larger static
+  // arrays (216 and more columns that fill their CTAs) runs on the cooperative
+  // grid.
   const void* fn = (const void*)k_hess_row<TO, true>;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(p.G);
@@ -1594,11 +1601,15 @@ static rr_status hess_res_launch(int64_t n, int64_t k, float* W, int64_t ldw, TO
   cfg.numAttrs = 1;
   bool cl = false;
   if (byrow && p.G <= kHessMaxCluster) {
-    RR_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    if (p.G > 8) RR_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-    int nc = 0;
-    cl = cudaOccupancyMaxActiveClusters(&nc, fn, &cfg) == cudaSuccess && nc >= 1;
-    if (!cl) (void)cudaGetLastError();
+    size_t most = 0;
+    RR_TRY(dynamic_smem_limit(fn, &most));
+    if (smem <= most) {
+      int nc = 0;
+      cl = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) == cudaSuccess &&
+           (p.G <= 8 || cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) &&
+           cudaOccupancyMaxActiveClusters(&nc, fn, &cfg) == cudaSuccess && nc >= 1;
+      if (!cl) (void)cudaGetLastError();
+    }
   }
   if (!cl) {
     fn = byrow ? (const void*)k_hess_row<TO, false> : (const void*)k_hess_res<TO>;

@@ -36,6 +36,18 @@ inline cudaStream_t as_stream(void* s) { return reinterpret_cast<cudaStream_t>(s
 
 int num_sms();
 
+// Most dynamic shared memory a launch of fn can have on the current device: what
+// a CTA can opt in to less the kernel's static shared memory.
+inline rr_status dynamic_smem_limit(const void* fn, size_t* most) {
+  int dev = 0, optin = 0;
+  cudaFuncAttributes at;
+  RR_CUDA(cudaGetDevice(&dev));
+  RR_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+  RR_CUDA(cudaFuncGetAttributes(&at, fn));
+  *most = (size_t)optin - at.sharedSizeBytes;
+  return RR_OK;
+}
+
 // ---------------------------------------------------------------------------
 // device helpers
 // ---------------------------------------------------------------------------
