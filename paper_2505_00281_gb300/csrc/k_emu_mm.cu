@@ -48,6 +48,7 @@
 // Every wait is bounded (2 s); on expiry the kernel records an error, drains
 // its copies and MMAs, frees its TMEM and returns.
 #include <algorithm>
+#include <climits>
 #include <type_traits>
 
 #include "rr_common.cuh"
@@ -866,7 +867,7 @@ __global__ void __launch_bounds__(256) k_emu_bslice(int64_t K, int64_t N, const 
 template <typename TS>
 __global__ void __launch_bounds__(256) k_emu_col_exp(int64_t n, const TS* __restrict__ X, int64_t ldx, int64_t rpc,
                                                      int* __restrict__ e) {
-  const int64_t j = blockIdx.y, r0 = (int64_t)blockIdx.x * rpc, r1 = min(n, r0 + rpc);
+  const int64_t j = blockIdx.x, r0 = (int64_t)blockIdx.y * rpc, r1 = min(n, r0 + rpc);
   const TS* x = X + j * ldx;
   int mx = kExpNone;
   for (int64_t i = r0 + threadIdx.x; i < r1; i += 8 * 256) {
@@ -877,7 +878,7 @@ __global__ void __launch_bounds__(256) k_emu_col_exp(int64_t n, const TS* __rest
     for (int u = 0; u < 8; ++u) mx = max(mx, exp_raw<TS>(v[u]));
   }
   mx = __reduce_max_sync(0xffffffffu, mx);
-  if (gridDim.x > 1) {
+  if (gridDim.y > 1) {
     if ((threadIdx.x & 31) == 0) atomicMax(e + j, mx);
     return;
   }
@@ -892,20 +893,21 @@ __global__ void __launch_bounds__(256) k_emu_col_exp(int64_t n, const TS* __rest
 }
 
 // Exponents of the largest entry of every row of a column-major block (lane =
-// row, 16 columns a thread, atomic maxima; e starts very negative).
+// row, 16 columns a thread at a time, atomic maxima; e starts very negative).
 template <typename TS>
 __global__ void __launch_bounds__(256) k_emu_row_exp(int64_t m, int64_t n, const TS* __restrict__ A, int64_t lda,
                                                      int* __restrict__ e) {
   const int64_t i = (int64_t)blockIdx.x * 32 + (threadIdx.x & 31);
-  const int64_t j0 = ((int64_t)blockIdx.y * 8 + (threadIdx.x >> 5)) * 16;
-  if (i >= m || j0 >= n) return;
-  typename Raw<TS>::R v[16];
+  if (i >= m) return;
+  int mx = INT_MIN;
+  for (int64_t j0 = ((int64_t)blockIdx.y * 8 + (threadIdx.x >> 5)) * 16; j0 < n; j0 += (int64_t)gridDim.y * 128) {
+    typename Raw<TS>::R v[16];
 #pragma unroll
-  for (int u = 0; u < 16; ++u) v[u] = j0 + u < n ? Raw<TS>::ld(A + i + (j0 + u) * lda) : 0;
-  int mx = kExpNone;
+    for (int u = 0; u < 16; ++u) v[u] = j0 + u < n ? Raw<TS>::ld(A + i + (j0 + u) * lda) : 0;
 #pragma unroll
-  for (int u = 0; u < 16; ++u) mx = max(mx, exp_raw<TS>(v[u]));
-  atomicMax(e + i, mx);
+    for (int u = 0; u < 16; ++u) mx = max(mx, exp_raw<TS>(v[u]));
+  }
+  if (mx > INT_MIN) atomicMax(e + i, mx);
 }
 
 // G (p x q) = the sum of the K ranges' partial tiles in a fixed order (+ G).
@@ -1054,7 +1056,7 @@ rr_status col_exps(cudaStream_t s, int32_t type, int64_t n, int64_t c, const voi
   int64_t chunks = col_exp_chunks(n, c);
   const int64_t rpc = (n + chunks - 1) / chunks;
   chunks = (n + rpc - 1) / rpc;
-  const dim3 g((unsigned)chunks, (unsigned)c);
+  const dim3 g((unsigned)c, (unsigned)chunks);
   switch (type) {
     case RR_F64: k_emu_col_exp<double><<<g, 256, 0, s>>>(n, (const double*)X, ldx, rpc, e); break;
     case RR_F32: k_emu_col_exp<float><<<g, 256, 0, s>>>(n, (const float*)X, ldx, rpc, e); break;
@@ -1066,7 +1068,8 @@ rr_status col_exps(cudaStream_t s, int32_t type, int64_t n, int64_t c, const voi
 }
 
 rr_status row_exps(cudaStream_t s, int32_t type, int64_t n, int64_t c, const void* X, int64_t ldx, int* e) {
-  const dim3 g((unsigned)((n + 31) / 32), (unsigned)((c + 127) / 128));
+  // (65535: the most blocks on y; the kernel strides over the columns beyond)
+  const dim3 g((unsigned)((n + 31) / 32), (unsigned)std::min<int64_t>((c + 127) / 128, 65535));
   switch (type) {
     case RR_F64: k_emu_row_exp<double><<<g, 256, 0, s>>>(n, c, (const double*)X, ldx, e); break;
     case RR_F32: k_emu_row_exp<float><<<g, 256, 0, s>>>(n, c, (const float*)X, ldx, e); break;
