@@ -288,7 +288,7 @@ rr_status rr_split_operator(int64_t m, int64_t n, const double* A, int64_t lda, 
  *   X (n x b, ld ldx) = S1 (n x p1, ld ld1) Y(0:p1, :) + S2 (n x p2, ld ld2) Y(p1:p1+p2, :)
  * with Y FP64 (p1+p2) x b (ld ldy), all column-major; S1, S2 of type t1, t2
  * (RR_F64, RR_F32 or RR_BF16); S2 may be NULL (p2 ignored).  FP64-accurate:
- * when p1+p2 is at most 512, b <= 256 and ws holds
+ * when p1+p2 is a multiple of 8 and at most 512, b <= 256 and ws holds
  * rr_lift_workspace_size(n, b, p1+p2) bytes, the product runs on the BF16
  * tensor cores through error-free 7-bit slices of both operands, formed on
  * chip (per-entry error below (p1+p2) 2^-47 max_k|S(i,k)| max_k|Y(k,j)|, each
@@ -439,12 +439,15 @@ rr_status rr_basis_builder(int32_t method, int32_t storage, int64_t n, int64_t k
 /* Projection products (Alg. 3: B = U^T A U, M = U^T U; Alg. 5: U^T A V,
  * U^T U, V^T V): G (p x q FP64, ld ldg) = X^T Y (+ G if accumulate) for tall
  * X (n x p) and Y (n x q) of types xtype/ytype (RR_F64, RR_F32, RR_BF16).
- * FP64-accurate: when n >= 64 the products run on the tensor cores from 7
- * column-scaled 7-bit slices of each operand, formed on chip, with exact FP32
- * sums over 448 rows at a time (error per entry below
- * 2^-47 n max|X(:,i)| max|Y(:,j)|); otherwise FP64 accumulation on the CUDA
- * cores.  Needs rr_gram_workspace_size(n, p, q) bytes (exponents and
- * deterministic split-K partials, reduced in a fixed order). */
+ * FP64-accurate: when n >= 64 and n % 8 == 0 the products run on the tensor
+ * cores from 7 column-scaled 7-bit slices of each operand, formed on chip, with
+ * exact FP32 sums over 448 rows at a time (error per entry below
+ * 2^-47 n max|X(:,i)| max|Y(:,j)|; FP64 subnormals count as zero); otherwise
+ * FP64 accumulation on the CUDA cores (n u64 of the sum of |X| |Y|).  With
+ * n >= 64 and p, q <= 4096 a column of X (Y) that holds an infinity or a NaN
+ * makes its row (column) of G NaN, in either arithmetic.  Needs
+ * rr_gram_workspace_size(n, p, q) bytes (exponents and deterministic split-K
+ * partials, reduced in a fixed order). */
 size_t rr_gram_workspace_size(int64_t n, int64_t p, int64_t q);
 rr_status rr_gram(int64_t n, int64_t p, int64_t q, int32_t xtype, const void* X, int64_t ldx,
                   int32_t ytype, const void* Y, int64_t ldy, double* G, int64_t ldg,

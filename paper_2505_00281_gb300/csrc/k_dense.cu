@@ -378,10 +378,18 @@ namespace rr {
 constexpr int GT = 32;      // output tile GT x GT
 constexpr int GROWS = 32;   // rows per smem stage
 
+// rr_gram gives a column with an infinity a NaN row (or column) of G whether or
+// not the row count is a multiple of 8, that is in slices or in FP64 arithmetic:
+// for the latter the infinity is read as a NaN (on the bit pattern: the FP64
+// units bound this kernel)
+__device__ __forceinline__ double inf_as_nan(double v, int on) {
+  return on && (__double2hiint(v) & 0x7FF00000) == 0x7FF00000 ? __longlong_as_double(0x7FF8000000000000ll) : v;
+}
+
 template <typename TX, typename TY, typename TA = double>
 __global__ void __launch_bounds__(256) k_gram_partial(
     int64_t n, int64_t p, int64_t q, const TX* __restrict__ X, int64_t ldx,
-    const TY* __restrict__ Y, int64_t ldy, int64_t rows_per_chunk, double* __restrict__ part) {
+    const TY* __restrict__ Y, int64_t ldy, int64_t rows_per_chunk, double* __restrict__ part, int inf_nan) {
   __shared__ TA Xs[GROWS][GT + 1];
   __shared__ TA Ys[GROWS][GT + 1];
   int64_t p0 = (int64_t)blockIdx.x * GT, q0 = (int64_t)blockIdx.y * GT;
@@ -394,8 +402,8 @@ __global__ void __launch_bounds__(256) k_gram_partial(
     for (int e = tid; e < GROWS * GT; e += 256) {
       int rr_ = e % GROWS, c = e / GROWS;
       int64_t row = rs + rr_;
-      Xs[rr_][c] = (row < r1 && p0 + c < p) ? LdAs<TA, TX>::get(X + row + (p0 + c) * ldx) : TA(0);
-      Ys[rr_][c] = (row < r1 && q0 + c < q) ? LdAs<TA, TY>::get(Y + row + (q0 + c) * ldy) : TA(0);
+      Xs[rr_][c] = (row < r1 && p0 + c < p) ? inf_as_nan(LdAs<TA, TX>::get(X + row + (p0 + c) * ldx), inf_nan) : TA(0);
+      Ys[rr_][c] = (row < r1 && q0 + c < q) ? inf_as_nan(LdAs<TA, TY>::get(Y + row + (q0 + c) * ldy), inf_nan) : TA(0);
     }
     __syncthreads();
 #pragma unroll 8
@@ -454,12 +462,12 @@ namespace rr {
 template <typename TX>
 static rr_status gram_dispatch_y(int32_t ytype, dim3 g, cudaStream_t s, int64_t n, int64_t p,
                                  int64_t q, const TX* X, int64_t ldx, const void* Y, int64_t ldy,
-                                 int64_t rpc, double* part) {
+                                 int64_t rpc, double* part, int inf_nan) {
   switch (ytype) {
-    case RR_F64: k_gram_partial<TX, double><<<g, 256, 0, s>>>(n, p, q, X, ldx, (const double*)Y, ldy, rpc, part); break;
-    case RR_F32: k_gram_partial<TX, float><<<g, 256, 0, s>>>(n, p, q, X, ldx, (const float*)Y, ldy, rpc, part); break;
-    case RR_BF16: k_gram_partial<TX, __nv_bfloat16><<<g, 256, 0, s>>>(n, p, q, X, ldx, (const __nv_bfloat16*)Y, ldy, rpc, part); break;
-    case RR_E4M3: k_gram_partial<TX, e4m3b_t><<<g, 256, 0, s>>>(n, p, q, X, ldx, (const e4m3b_t*)Y, ldy, rpc, part); break;
+    case RR_F64: k_gram_partial<TX, double><<<g, 256, 0, s>>>(n, p, q, X, ldx, (const double*)Y, ldy, rpc, part, inf_nan); break;
+    case RR_F32: k_gram_partial<TX, float><<<g, 256, 0, s>>>(n, p, q, X, ldx, (const float*)Y, ldy, rpc, part, inf_nan); break;
+    case RR_BF16: k_gram_partial<TX, __nv_bfloat16><<<g, 256, 0, s>>>(n, p, q, X, ldx, (const __nv_bfloat16*)Y, ldy, rpc, part, inf_nan); break;
+    case RR_E4M3: k_gram_partial<TX, e4m3b_t><<<g, 256, 0, s>>>(n, p, q, X, ldx, (const e4m3b_t*)Y, ldy, rpc, part, inf_nan); break;
     default: return RR_ERR_ARG;
   }
   return RR_OK;
@@ -653,13 +661,14 @@ extern "C" rr_status rr_gram(int64_t n, int64_t p, int64_t q, int32_t xtype, con
   int64_t rpc = (n + chunks - 1) / chunks;
   chunks = (n + rpc - 1) / rpc;
   double* part = (double*)ws;
+  const int inf_nan = n >= 64 && n % 8 != 0 && p <= 4096 && q <= 4096;
   dim3 g((unsigned)((p + GT - 1) / GT), (unsigned)((q + GT - 1) / GT), (unsigned)chunks);
   rr_status st;
   switch (xtype) {
-    case RR_F64: st = gram_dispatch_y<double>(ytype, g, s, n, p, q, (const double*)X, ldx, Y, ldy, rpc, part); break;
-    case RR_F32: st = gram_dispatch_y<float>(ytype, g, s, n, p, q, (const float*)X, ldx, Y, ldy, rpc, part); break;
-    case RR_BF16: st = gram_dispatch_y<__nv_bfloat16>(ytype, g, s, n, p, q, (const __nv_bfloat16*)X, ldx, Y, ldy, rpc, part); break;
-    case RR_E4M3: st = gram_dispatch_y<e4m3b_t>(ytype, g, s, n, p, q, (const e4m3b_t*)X, ldx, Y, ldy, rpc, part); break;
+    case RR_F64: st = gram_dispatch_y<double>(ytype, g, s, n, p, q, (const double*)X, ldx, Y, ldy, rpc, part, inf_nan); break;
+    case RR_F32: st = gram_dispatch_y<float>(ytype, g, s, n, p, q, (const float*)X, ldx, Y, ldy, rpc, part, inf_nan); break;
+    case RR_BF16: st = gram_dispatch_y<__nv_bfloat16>(ytype, g, s, n, p, q, (const __nv_bfloat16*)X, ldx, Y, ldy, rpc, part, inf_nan); break;
+    case RR_E4M3: st = gram_dispatch_y<e4m3b_t>(ytype, g, s, n, p, q, (const e4m3b_t*)X, ldx, Y, ldy, rpc, part, inf_nan); break;
     default: return RR_ERR_ARG;
   }
   if (st != RR_OK) return st;
@@ -754,10 +763,10 @@ extern "C" rr_status rr_gram_noalloc(int64_t n, int64_t p, int64_t q, int32_t xt
   dim3 g((unsigned)((p + GT - 1) / GT), (unsigned)((q + GT - 1) / GT), (unsigned)chunks);
   rr_status st;
   switch (xtype) {
-    case RR_F64: st = gram_dispatch_y<double>(ytype, g, s, n, p, q, (const double*)X, ldx, Y, ldy, rpc, scratch); break;
-    case RR_F32: st = gram_dispatch_y<float>(ytype, g, s, n, p, q, (const float*)X, ldx, Y, ldy, rpc, scratch); break;
-    case RR_BF16: st = gram_dispatch_y<__nv_bfloat16>(ytype, g, s, n, p, q, (const __nv_bfloat16*)X, ldx, Y, ldy, rpc, scratch); break;
-    case RR_E4M3: st = gram_dispatch_y<e4m3b_t>(ytype, g, s, n, p, q, (const e4m3b_t*)X, ldx, Y, ldy, rpc, scratch); break;
+    case RR_F64: st = gram_dispatch_y<double>(ytype, g, s, n, p, q, (const double*)X, ldx, Y, ldy, rpc, scratch, 0); break;
+    case RR_F32: st = gram_dispatch_y<float>(ytype, g, s, n, p, q, (const float*)X, ldx, Y, ldy, rpc, scratch, 0); break;
+    case RR_BF16: st = gram_dispatch_y<__nv_bfloat16>(ytype, g, s, n, p, q, (const __nv_bfloat16*)X, ldx, Y, ldy, rpc, scratch, 0); break;
+    case RR_E4M3: st = gram_dispatch_y<e4m3b_t>(ytype, g, s, n, p, q, (const e4m3b_t*)X, ldx, Y, ldy, rpc, scratch, 0); break;
     default: return RR_ERR_ARG;
   }
   if (st != RR_OK) return st;

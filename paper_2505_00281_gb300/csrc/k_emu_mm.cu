@@ -1187,14 +1187,16 @@ size_t lift_emu_bytes(int64_t n, int64_t b, int64_t K) {
   return 2 * align_up((size_t)n * 4) + blob_bytes(K, b, 7) + blob_bytes(kKB, b, 7) + 256;
 }
 
-// *done = false (nothing launched) when the shape is outside this path.
+// *done = false (nothing launched) when the shape is outside this path.  K that
+// is no multiple of 8 is left to FP64 arithmetic, whose error is relative to the
+// terms summed and not to the largest entries of rows and columns.
 rr_status lift_emu(cudaStream_t s, int64_t n, int64_t b, int32_t t1, const void* S1, int64_t ld1, int64_t p1,
                    int32_t t2, const void* S2, int64_t ld2, int64_t p2, const double* Y, int64_t ldy, double* X,
                    int64_t ldx, void* mem, size_t mem_bytes, bool* done) {
   *done = false;
   if (!S2) p2 = 0;
   const int64_t K = p1 + p2;
-  if (!mem || n <= 0 || n > 0x7fffff00ll || b <= 0 || b > 256 || K > 512 || p1 <= 0 ||
+  if (!mem || n <= 0 || n > 0x7fffff00ll || b <= 0 || b > 256 || K % 8 || K > 512 || p1 <= 0 ||
       ((uintptr_t)mem & 15))
     return RR_OK;
   if (mem_bytes < lift_emu_bytes(n, b, K)) return RR_OK;
@@ -1232,8 +1234,9 @@ rr_status lift_emu(cudaStream_t s, int64_t n, int64_t b, int32_t t1, const void*
 // ---------------------------------------------------------------------------
 // Gram products G = X^T Y (X n x p, Y n x q, any storage type).
 // ---------------------------------------------------------------------------
+// (Row counts that are no multiple of 8 stay in FP64 arithmetic, as in the lift.)
 bool emu_gram_supported(int64_t n, int64_t p, int64_t q) {
-  return n >= 64 && p >= 1 && q >= 1 && p <= 4096 && q <= 4096 && n <= ((int64_t)1 << 30);
+  return n >= 64 && n % 8 == 0 && p >= 1 && q >= 1 && p <= 4096 && q <= 4096 && n <= ((int64_t)1 << 30);
 }
 
 // Tiles: rows in blocks of 128 of X's columns; a remainder of at most 64 rows
