@@ -1860,17 +1860,18 @@ static rr_status hess_blocked(int64_t n, int64_t k, float* W, int64_t ldw, TO* Q
 }
 
 // The FP32 process of a whole block: resident where it fits the CTAs' shared
-// memory, blocked (panels of 32, their columns resident) where it does not, and
-// the right-looking kernel for a single CTA (the batched solver's concurrent
-// problems), for rows beyond its candidate word and where not even one panel
-// column fits.
+// memory, blocked where it does not (panels of 32 with as many resident columns
+// as fit; panels of 16 on W in memory past 8.7 million rows, where not even one
+// column is resident: 10M x 96 took 380 ms as one right-looking panel), and the
+// right-looking kernel for a single CTA (the batched solver's concurrent
+// problems), for rows beyond its candidate word and for one such panel.
 template <typename TO>
 static rr_status hess_f32(int64_t n, int64_t k, float* W, int64_t ldw, TO* Q, int64_t ldq, int* piv, double tol,
                           void* ws, size_t ws_bytes, cudaStream_t s, int max_grid) {
   const HessPlan p = hess_plan(n, k);
-  if (max_grid == 1 || n == 0 || n >= (int64_t)kNoRow || p.kr < 1)
+  if (max_grid == 1 || n == 0 || n >= (int64_t)kNoRow || (p.kr < 1 && k <= 16))
     return hess_launch<float, TO>(n, k, W, ldw, Q, ldq, piv, tol, ws, ws_bytes, s, max_grid);
-  if (p.kr < k) return hess_blocked<TO>(n, k, W, ldw, Q, ldq, piv, tol, kPanelMax, ws, ws_bytes, s);
+  if (p.kr < k) return hess_blocked<TO>(n, k, W, ldw, Q, ldq, piv, tol, p.kr < 1 ? 16 : kPanelMax, ws, ws_bytes, s);
   const size_t base = hess_ws_bytes<float>(k, num_sms());
   if (!ws || ws_bytes < base + hess_blocked_extra(k)) return RR_ERR_WORKSPACE;
   RR_CUDA(cudaMemsetAsync(ws, 0, 512, s));  // err + barrier
