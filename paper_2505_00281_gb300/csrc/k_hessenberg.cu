@@ -1735,7 +1735,7 @@ __global__ void __launch_bounds__(256) k_hess_trail(int64_t n, int r, int nt, co
   extern __shared__ __align__(16) float sw[];  // [nt][R] -w
   for (int e = threadIdx.x; e < R * nt; e += blockDim.x) {
     const int c = e / R, j = e % R;
-    sw[e] = j < r ? -w[j * (size_t)wld + c] : 0.f;
+    sw[e] = -(j < r ? w[j * (size_t)wld + c] : 0.f);  // (padding: -0 times its zero entries, x + -0 = x)
   }
   __syncthreads();
   auto ld = [&](const float* p, bool two) -> float2 {
