@@ -755,8 +755,7 @@ static rr_status hess_launch(int64_t n, int64_t k, T* W, int64_t ldw, TO* Q, int
   const size_t fixed = (packed ? 3 : 2) * (size_t)k * sizeof(T) + 16;  // thresholds, weights, alignment
   if ((size_t)ldv * k * sizeof(T) <= kSlabLimit && (size_t)ldv * k * sizeof(T) + fixed <= 220 * 1024) slab = 1;
   size_t smem = fixed + (slab ? (size_t)ldv * k * sizeof(T) : 0);
-  if (smem > 48 * 1024)
-    RR_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  RR_TRY(allow_dynamic_smem(fn, smem));
   if (ws_bytes < hess_ws_bytes<T>(k, G) || !ws) return RR_ERR_WORKSPACE;
   Arena ar(ws, ws_bytes);
   HessWs<T> h;
@@ -1601,12 +1600,11 @@ static rr_status hess_res_launch(int64_t n, int64_t k, float* W, int64_t ldw, TO
   cfg.numAttrs = 1;
   bool cl = false;
   if (byrow && p.G <= kHessMaxCluster) {
-    size_t most = 0;
-    RR_TRY(dynamic_smem_limit(fn, &most));
-    if (smem <= most) {
+    bool fits = false;
+    RR_TRY(allow_dynamic_smem(fn, smem, &fits));
+    if (fits) {
       int nc = 0;
-      cl = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) == cudaSuccess &&
-           (p.G <= 8 || cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) &&
+      cl = (p.G <= 8 || cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) &&
            cudaOccupancyMaxActiveClusters(&nc, fn, &cfg) == cudaSuccess && nc >= 1;
       if (!cl) (void)cudaGetLastError();
     }
@@ -1614,7 +1612,7 @@ static rr_status hess_res_launch(int64_t n, int64_t k, float* W, int64_t ldw, TO
   if (!cl) {
     fn = byrow ? (const void*)k_hess_row<TO, false> : (const void*)k_hess_res<TO>;
     cfg.attrs = at;
-    RR_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    RR_TRY(allow_dynamic_smem(fn, smem));
   }
   Arena ar(mem, hess_res_bytes(kmem));
   HessRes h;
@@ -1798,7 +1796,7 @@ static rr_status hess_trail(int64_t n, int r, int nt, const float* L, float* T, 
     const int nc = std::min(nt - c0, ncmax);
     const size_t sm = (size_t)R * nc * sizeof(float);
     auto go = [&](auto fn) -> rr_status {
-      if (sm > 48 * 1024) RR_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+      RR_TRY(allow_dynamic_smem((const void*)fn, sm));
       fn<<<g, 256, sm, s>>>(n, r, nc, L, T + (int64_t)c0 * ldw, ldw, wts + c0, nt, -0.0f);
       return check_launch("hessenberg trailing update");
     };

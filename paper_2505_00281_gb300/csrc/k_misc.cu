@@ -232,7 +232,7 @@ static rr_status launch_sub_lowrank32_full(cudaStream_t s, int64_t n, int64_t b,
                                            int64_t ldx, const double* K, int64_t ldk, float* T, int64_t ldt) {
   const size_t smem =
       ((((size_t)p * (16 * CT + 2) + 3) & ~(size_t)3) + (size_t)kSLF_K * kSLF_M + (size_t)b * kSLF_M) * sizeof(float);
-  RR_CUDA(cudaFuncSetAttribute(k_sub_lowrank32_full<CT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  RR_TRY(allow_dynamic_smem((const void*)k_sub_lowrank32_full<CT>, smem));
   const int64_t tiles = (n + kSLF_M - 1) / kSLF_M;
   const int64_t grid = tiles < num_sms() ? tiles : num_sms();
   k_sub_lowrank32_full<CT><<<(unsigned)grid, 256, smem, s>>>(n, (int)b, (int)p, X, ldx, K, ldk, T, ldt);

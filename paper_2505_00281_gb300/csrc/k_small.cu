@@ -352,8 +352,7 @@ static size_t shift_trial_smem(int b) { return (size_t)b * (b + 1) / 2 * sizeof(
 static rr_status eig_shift(cudaStream_t s, int b, double* C, const int* dropped, double* sh, int* ok, double* mu) {
   k_eig_prep<<<1, kSmallThreads, 0, s>>>(b, C, dropped, sh);
   const size_t sm = shift_trial_smem(b);
-  if (sm > 48 * 1024)
-    RR_CUDA(cudaFuncSetAttribute(k_shift_trials, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+  RR_TRY(allow_dynamic_smem((const void*)k_shift_trials, sm));
   k_shift_trials<<<kShiftTrials, kShiftThreads, sm, s>>>(b, C, dropped, sh, ok);
   k_shift_pick<<<1, 256, 0, s>>>(b, C, dropped, sh, ok, 1, mu);
   note_launches(2);  // with check_launch's one: prep, the trials, the pick
@@ -1653,13 +1652,11 @@ static void whiten(cudaStream_t s, int b, const double* G, const WhitenScratch& 
   const int g1 = (b * b + 255) / 256;
   if (b <= kCT * kCTMax) {
     const size_t sm = chol_blocked_smem(b);
-    if (sm > 48 * 1024)
-      cudaFuncSetAttribute(k_chol_inv_blocked, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    (void)allow_dynamic_smem((const void*)k_chol_inv_blocked, sm);  // (a refusal shows in the launch check)
     k_chol_inv_blocked<<<1, kChThreads, sm, s>>>(b, G, b, dropped, w.W1);
   } else {
     const size_t sm = ((size_t)b * (b + 1) / 2 + 2 * (size_t)b) * sizeof(float);
-    if (sm > 48 * 1024)
-      cudaFuncSetAttribute(k_chol_inv_f32, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    (void)allow_dynamic_smem((const void*)k_chol_inv_f32, sm);
     k_chol_inv_f32<<<1, kSmallThreads, sm, s>>>(b, G, b, dropped, w.W1);
   }
   // every step writes the other buffer (the products never run in place);
@@ -1788,8 +1785,7 @@ static rr_status launch_bj(cudaStream_t s, int r, int cpad, int w, int P, float*
   if (P <= kBJMaxCluster && csm <= 220 * 1024) {
     // one cluster: columns stay in shared memory, no global barrier
     const void* fn = (const void*)k_block_jacobi_cl;
-    if (csm > 48 * 1024)
-      RR_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)csm));
+    RR_TRY(allow_dynamic_smem(fn, csm));
     if (2 * P > 8) RR_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(2 * P);
@@ -1816,8 +1812,7 @@ static rr_status launch_bj(cudaStream_t s, int r, int cpad, int w, int P, float*
   }
   const size_t smem = bj_smem(r, cpad, w);
   const void* fn = (const void*)k_block_jacobi;
-  if (smem > 48 * 1024)
-    RR_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  RR_TRY(allow_dynamic_smem(fn, smem));
   RR_CUDA(cudaMemsetAsync(ws.rot, 0, 64 * sizeof(int), s));
   RR_CUDA(cudaMemsetAsync(ws.bar, 0, sizeof(GridBarrier), s));
   int ld = r, ldv = cpad;
@@ -2466,8 +2461,7 @@ static rr_status jacobi_svd(cudaStream_t s, int r, int c, const double* C, Penci
   RR_TRY(launch_bj(s, r, cpad, ww, P, w.M32, w.V32, 1e-4f, 15, w, fl));
   k_v32_to_64<<<g, 256, 0, s>>>(c, cpad, w.V32, w.V);
   const size_t csm = cluster_smem(c);
-  if (csm > 48 * 1024)
-    RR_CUDA(cudaFuncSetAttribute(k_cluster_rot, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)csm));
+  RR_TRY(allow_dynamic_smem((const void*)k_cluster_rot, csm));
   constexpr int kRefineSteps = 4;
   for (int it = 0; it < kRefineSteps; ++it) {
     gemm_small(s, 0, 0, r, c, c, 1.0, C, r, w.V, c, 0.0, w.Mp, r);          // N = C V

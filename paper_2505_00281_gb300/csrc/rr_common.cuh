@@ -36,15 +36,26 @@ inline cudaStream_t as_stream(void* s) { return reinterpret_cast<cudaStream_t>(s
 
 int num_sms();
 
-// Most dynamic shared memory a launch of fn can have on the current device: what
-// a CTA can opt in to less the kernel's static shared memory.
-inline rr_status dynamic_smem_limit(const void* fn, size_t* most) {
-  int dev = 0, optin = 0;
+// Lets fn be launched with `bytes` of dynamic shared memory.  The limit is an
+// attribute of the function, shared by every thread of the process: it is raised
+// to the most a launch can have (what a CTA can opt in to less the kernel's
+// static part) and never lowered, so that threads launching blocks of different
+// sizes do not take it from one another.  More than that is an error, or with
+// `fits` given the answer false.
+inline rr_status allow_dynamic_smem(const void* fn, size_t bytes, bool* fits = nullptr) {
   cudaFuncAttributes at;
+  RR_CUDA(cudaFuncGetAttributes(&at, fn));
+  if (fits) *fits = true;
+  if (bytes <= (size_t)at.maxDynamicSharedSizeBytes) return RR_OK;
+  int dev = 0, optin = 0;
   RR_CUDA(cudaGetDevice(&dev));
   RR_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-  RR_CUDA(cudaFuncGetAttributes(&at, fn));
-  *most = (size_t)optin - at.sharedSizeBytes;
+  const size_t most = (size_t)optin - at.sharedSizeBytes;
+  if (bytes > most && fits) {
+    *fits = false;
+    return RR_OK;
+  }
+  RR_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(bytes > most ? bytes : most)));
   return RR_OK;
 }
 
