@@ -444,8 +444,9 @@ rr_status rr_basis_builder(int32_t method, int32_t storage, int64_t n, int64_t k
  * exact FP32 sums over 448 rows at a time (error per entry below
  * 2^-47 n max|X(:,i)| max|Y(:,j)|; FP64 subnormals count as zero); otherwise
  * FP64 accumulation on the CUDA cores (n u64 of the sum of |X| |Y|).  With
- * n >= 64 and p, q <= 4096 a column of X (Y) that holds an infinity or a NaN
- * makes its row (column) of G NaN, in either arithmetic.  Needs
+ * n >= 64 and p <= 4096 (and q <= 4096 where n % 8 != 0) a column of X (Y) that
+ * holds an infinity or a NaN makes its row (column) of G NaN, in either
+ * arithmetic.  Needs
  * rr_gram_workspace_size(n, p, q) bytes (exponents and deterministic split-K
  * partials, reduced in a fixed order). */
 size_t rr_gram_workspace_size(int64_t n, int64_t p, int64_t q);

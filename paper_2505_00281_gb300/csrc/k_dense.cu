@@ -445,14 +445,19 @@ static int64_t gram_chunks(int64_t n, int64_t p, int64_t q) {
   int64_t c = want < maxc ? want : maxc;
   return c < 1 ? 1 : c;
 }
+
+// columns of Y that one launch of the tensor-core path takes: a wider Y goes in
+// column chunks
+constexpr int64_t kGramCols = 4096;
 }  // namespace rr
 
 // Workspace: the SIMT path's split-K partials, or the tensor-core path's
 // exponents and partial tiles when the shape qualifies
 extern "C" size_t rr_gram_workspace_size(int64_t n, int64_t p, int64_t q) {
   size_t b = align_up((size_t)gram_chunks(n, p, q) * p * q * sizeof(double)) + 256;
-  if (emu_gram_supported(n, p, q)) {
-    const size_t e = emu_gram_bytes(n, p, q);
+  const int64_t qe = q < kGramCols ? q : kGramCols;
+  if (emu_gram_supported(n, p, qe)) {
+    const size_t e = emu_gram_bytes(n, p, qe);
     if (e > b) b = e;
   }
   return b;
@@ -654,14 +659,22 @@ extern "C" rr_status rr_gram(int64_t n, int64_t p, int64_t q, int32_t xtype, con
   }
   // FP64-accurate products on the tensor cores when the shape qualifies and
   // the workspace holds the partial tiles
-  if (emu_gram_supported(n, p, q) && ws && ws_bytes >= emu_gram_bytes(n, p, q))
-    return emu_gram(s, n, p, q, xtype, X, ldx, ytype, Y, ldy, G, ldg, accumulate, ws, ws_bytes);
+  const int64_t qe = q < kGramCols ? q : kGramCols;
+  if (emu_gram_supported(n, p, qe) && ws && ws_bytes >= emu_gram_bytes(n, p, qe)) {
+    const size_t ys = dtype_size(ytype);
+    for (int64_t j0 = 0; j0 < q; j0 += kGramCols) {
+      const int64_t qc = std::min<int64_t>(kGramCols, q - j0);
+      RR_TRY(emu_gram(s, n, p, qc, xtype, X, ldx, ytype, (const char*)Y + (size_t)j0 * ldy * ys, ldy, G + j0 * ldg,
+                      ldg, accumulate, ws, ws_bytes));
+    }
+    return RR_OK;
+  }
   int64_t chunks = gram_chunks(n, p, q);
   if (ws_bytes < (size_t)chunks * p * q * sizeof(double) || !ws) return RR_ERR_WORKSPACE;
   int64_t rpc = (n + chunks - 1) / chunks;
   chunks = (n + rpc - 1) / rpc;
   double* part = (double*)ws;
-  const int inf_nan = n >= 64 && n % 8 != 0 && p <= 4096 && q <= 4096;
+  const int inf_nan = n >= 64 && n % 8 != 0 && p <= 4096 && q <= kGramCols;
   dim3 g((unsigned)((p + GT - 1) / GT), (unsigned)((q + GT - 1) / GT), (unsigned)chunks);
   rr_status st;
   switch (xtype) {
