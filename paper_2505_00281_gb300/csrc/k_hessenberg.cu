@@ -1529,8 +1529,14 @@ __global__ void __launch_bounds__(kRowThreads + 32 * kMaxPoll, 1) k_hess_row(
 
 // Dynamic shared memory a plan may ask for: the 227 KB a CTA can have less 2 KB
 // for the static arrays of the cooperative kernels (1040 bytes, -Xptxas -v).  The
-// cluster form holds 2560 bytes more of them: its launch checks that it fits.
+// cluster form holds 2560 bytes more of them: 228848 bytes.
 constexpr int64_t kHessSmem = 225 * 1024;
+constexpr int64_t kHessClusterSmem = kHessSmem + 1008 - 2560;
+
+// ... of k resident columns: slab, thresholds, trailing weights
+static size_t hess_res_smem(int64_t rpc, int64_t k) {
+  return (size_t)(rpc | 1) * 4 * k + 4 * (size_t)k + 32 + (k > kPw ? (size_t)(k - kPw) * kPw * 4 : 0);
+}
 
 // rows per CTA, CTAs and the columns that fit in shared memory
 struct HessPlan {
@@ -1543,6 +1549,12 @@ static HessPlan hess_plan(int64_t n, int64_t k) {
   int64_t G = (n + 255) / 256;
   const int64_t fit = (int64_t)((kHessSmem - 32 - 36 * k) / (4 * k)) - 1;
   if (fit >= 1 && (n + G - 1) / G > fit) G = (n + fit - 1) / fit;
+  // one CTA more where the block then fits one cluster (the exchange through
+  // distributed shared memory: 1024 x 216 takes 0.59 ms on 4 CTAs of the
+  // cooperative grid, 1024 x 200 0.46 in one cluster)
+  int64_t gc = G;
+  while (gc <= kHessMaxCluster && hess_res_smem((n + gc - 1) / gc, k) > (size_t)kHessClusterSmem) ++gc;
+  if (gc <= kHessMaxCluster) G = gc;
   if (G > num_sms()) G = num_sms();
   if (G > 32 * kMaxPoll) G = 32 * kMaxPoll;
   if (G < 1) G = 1;
@@ -1571,7 +1583,7 @@ template <typename TO>
 static rr_status hess_res_launch(int64_t n, int64_t k, float* W, int64_t ldw, TO* Q, int64_t ldq, int* piv, float tol,
                                  const HessPlan& p, void* ws, void* mem, int64_t kmem, int tag0,
                                  const float* colmax_ext, cudaStream_t s) {
-  const size_t smem = (size_t)(p.rpc | 1) * 4 * k + 4 * (size_t)k + 32 + (k > kPw ? (size_t)(k - kPw) * kPw * 4 : 0);
+  const size_t smem = hess_res_smem(p.rpc, k);
   const bool byrow = p.rpc <= kRowThreads;
   int rt = byrow ? (p.rpc + 31) / 32 * 32 : kRowThreads;
   const unsigned threads = rt + 32 * ((p.G + 31) / 32);
