@@ -73,7 +73,9 @@ template <int T>
 struct EmuConst {
   static constexpr int kg = T == 7 ? 14 : 11;      // stages of one exact FP32 accumulation
   static constexpr int base_shift = 7 * (T - 7) + 3;  // bits dropped from a group's exact integer sum
-  static constexpr int max_w = T == 7 ? 64 : 16;   // tile columns: T max_w <= 512 and the shared memory
+  // tile columns: T max_w <= 512, and the shared memory: 213 KB for 32 columns of
+  // T = 9 (16384 x 4096 x 128 with 16: 2.40 ms, every column tile slices A again)
+  static constexpr int max_w = T == 7 ? 64 : 32;
 };
 
 // stages of an accumulation group: nst stages in groups of about one size
