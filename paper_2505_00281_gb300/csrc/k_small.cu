@@ -2198,6 +2198,14 @@ constexpr double kCoupleNoise = 1e-13;
 // pair at residual 4e-10.
 constexpr double kSepGap = 1e-3;
 constexpr int kClMax = 32;          // largest cluster resolved as one block
+// A run of more than kClMax close values is cut into clusters, and pairs across a
+// cut keep angles of any size.  Applied together with everything else they
+// compose to anything but a rotation: the null space of a pencil of low rank or
+// of one with far more columns than rows (36 x 100: 64 zero values) took V to
+// 1e50 in four steps.  They are left alone instead (twice kBigAngle: the link
+// test is in FP32), so V stays orthogonal and every value outside the run
+// converges as ever; values within such a run stay as the Jacobi left them.
+constexpr double kMaxAngle = 2 * kBigAngle;
 constexpr int kClWarps = 8;         // clusters resolved at once
 
 __device__ __forceinline__ double oa_coupling(const double* K, const double* T, int c, int i, int j,
@@ -2225,6 +2233,7 @@ __global__ void k_oa_update(int c, const double* __restrict__ K, const double* _
     const double cij = oa_coupling(K, T, c, i, j, li, lj);
     const double big = fmax(fabs(li), fabs(lj));
     if (fabs(lj - li) > kSepGap * big || fabs(cij) > kCoupleNoise * big) wij = 0.5 * atan(2.0 * cij / (lj - li));
+    if (fabs(wij) > kMaxAngle) wij = 0.0;
   }
   F1[e] = f + wij;
   Wout[e] = wij;
