@@ -291,9 +291,10 @@ rr_status rr_split_operator(int64_t m, int64_t n, const double* A, int64_t lda, 
  * when p1+p2 is a multiple of 8 and at most 512, b <= 256 and ws holds
  * rr_lift_workspace_size(n, b, p1+p2) bytes, the product runs on the BF16
  * tensor cores through error-free 7-bit slices of both operands, formed on
- * chip (per-entry error below (p1+p2) 2^-47 max_k|S(i,k)| max_k|Y(k,j)|, each
- * block of S with its own row maxima); otherwise in FP64 arithmetic.  RR_ERR_ARG: negative sizes, p1 < 1, b < 1, bad type or NULL
- * pointers. */
+ * chip (per-entry error below (p1+p2) 2^-45 max_k|S(i,k)| max_k|Y(k,j)|, each
+ * block of S with its own row maxima, and FP64 roundings of the sum; see
+ * rr_gemm_f64_emulated); otherwise in FP64 arithmetic.  RR_ERR_ARG: negative
+ * sizes, p1 < 1, b < 1, bad type or NULL pointers. */
 size_t rr_lift_workspace_size(int64_t n, int64_t b, int64_t K);
 rr_status rr_lift(int64_t n, int64_t b, int32_t t1, const void* S1, int64_t ld1, int64_t p1,
                   int32_t t2, const void* S2, int64_t ld2, int64_t p2, const double* Y, int64_t ldy,
@@ -336,9 +337,12 @@ rr_status rr_gemm_f64(int32_t trans, int64_t M, int64_t N, int64_t K, const doub
  * scaled by powers of two and cut on chip into integer BF16 slices of 7 bits
  * (7 of them for `slices` 1..8, 9 for 9 and 10); the pair products are exact
  * in the FP32 tensor-core accumulator (448 columns of K at a time) and are
- * combined in 64-bit integers.  With 7 slices the result agrees with FP64
- * arithmetic to about 2^-54 of |op(A)| |B|.  N <= 256; m and n must be
- * multiples of 8.  Needs rr_gemm_f64_emulated_workspace_size bytes (exponents
+ * combined in 64-bit integers.  Error per entry below
+ *   K 2^-45 max_k |op(A)(i,k)| max_k |B(k,j)|      (9 slices: K 2^-59 ...)
+ * and FP64 roundings of the sum: per term, relative to the two powers of two
+ * (each up to twice its largest entry), the slices' remainders are 2 2^-50 and
+ * the dropped pairs p + q = 9 are 6 2^-51, the later ones less.  N <= 256; m and
+ * n must be multiples of 8.  Needs rr_gemm_f64_emulated_workspace_size bytes (exponents
  * and the slices of B). */
 size_t rr_gemm_f64_emulated_workspace_size(int32_t trans, int64_t M, int64_t N, int64_t K,
                                            int32_t slices);
@@ -442,7 +446,8 @@ rr_status rr_basis_builder(int32_t method, int32_t storage, int64_t n, int64_t k
  * FP64-accurate: when n >= 64 and n % 8 == 0 the products run on the tensor
  * cores from 7 column-scaled 7-bit slices of each operand, formed on chip, with
  * exact FP32 sums over 448 rows at a time (error per entry below
- * 2^-47 n max|X(:,i)| max|Y(:,j)|; FP64 subnormals count as zero); otherwise
+ * 2^-45 n max|X(:,i)| max|Y(:,j)| and FP64 roundings of the sum; FP64
+ * subnormals count as zero); otherwise
  * FP64 accumulation on the CUDA cores (n u64 of the sum of |X| |Y|).  With
  * n >= 64 and p <= 4096 (and q <= 4096 where n % 8 != 0) a column of X (Y) that
  * holds an infinity or a NaN makes its row (column) of G NaN, in either

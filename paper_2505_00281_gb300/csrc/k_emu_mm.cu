@@ -18,8 +18,10 @@
 // and one integer-to-double conversion per element ends the tile.
 //   T = 7 keeps more than the 8 slices of 6 bits used before it (remainder
 // 2^-50 against 2^-49, dropped pairs 6 2^-51 against 7 2^-50 of the row and
-// column scales) with 28 pair products instead of 36.  T = 9 serves callers
-// that ask for 9 or 10 slices of 6 bits.
+// column scales) with 28 pair products instead of 36.  A term errs by less than
+// 5.1 2^-50 of the two scales, each up to twice its largest entry: 2^-45 of the
+// largest entries.  T = 9 serves callers that ask for 9 or 10 slices of 6 bits
+// (1.6 2^-62 of the scales, 2^-59 of the largest entries).
 //
 // Why slicing belongs in this kernel: sliced operands are 14 bytes an entry,
 // written once and read back per tile, which bounded every use (a 1M x 160
