@@ -499,14 +499,14 @@ rr_status rr_gram_noalloc(int64_t n, int64_t p, int64_t q, int32_t xtype, const 
  *   Lu^-1 B Lv^-T by one-sided Jacobi (equivalent to the positive half of
  *   the 2x2 block pencil).
  * Sizes up to 335 x 335 (RR_ERR_ARG above).
- * Accuracy: values to b u64 of the largest, vectors orthonormal to b u64 (a
- * left vector of value sigma to b u64 s_1 / sigma), with one limit: values
- * that one-sided Jacobi in FP32 cannot tell apart (within 1e-4 of each other
+ * Accuracy: values to b u64 of the largest, right vectors orthonormal to b u64
+ * (a left vector of value sigma to b u64 s_1 / sigma), with one limit.  Values
+ * that one-sided Jacobi in FP32 leaves together (closer than about 1e-4
  * relatively, or below about 1e-5 of the largest, zeros included) are separated
- * in FP64 in groups of at most 32.  Where more than 32 lie together, the values
- * of that group are good to 1e-5 of the largest, its right vectors orthonormal
- * to about 1e-5 and its left vectors not orthogonal among themselves; every
- * value and vector outside it is as accurate as stated.
+ * in FP64 in groups of at most 32, and larger groups in part: where more than 32
+ * lie together, the group's values may be off by 1e-5 of the largest, its right
+ * vectors orthonormal to 1e-2 only and its left vectors not orthogonal among
+ * themselves.  Every value and vector outside it is as accurate as stated.
  * Both need rr_pencil_workspace_size(b1, b2) bytes of workspace and
  * synchronise nothing (dropped counts are read only when dropped != NULL,
  * which synchronises). */

@@ -1514,7 +1514,7 @@ struct PencilWs {
   double* cond;                        // [4] condition estimates of the whitened Grams, drop counts
   float *L32, *Li32, *M32, *V32, *fs;  // fs: [0] Jacobi norm floor, [1] scale
   float *Hq, *tq;                      // QR preconditioner: reflectors (c x c), taus
-  int *drop1, *drop2, *order, *nvalid, *rot, *err, *sweeps, *cid, *cst;
+  int *drop1, *drop2, *order, *nvalid, *rot, *err, *sweeps, *cid, *cst, *wild;
   GridBarrier* bar;
 };
 
@@ -1582,6 +1582,7 @@ static bool carve_pencil(Arena& ar, int b1, int b2, PencilWs& w) {
   w.sweeps = ar.take<int>(2);
   w.cid = ar.take<int>(cp);
   w.cst = ar.take<int>(cp + 1);
+  w.wild = ar.take<int>(cp);
   w.bar = ar.take<GridBarrier>(1);
   return !ar.overflow;
 }
@@ -2199,13 +2200,17 @@ constexpr double kCoupleNoise = 1e-13;
 constexpr double kSepGap = 1e-3;
 constexpr int kClMax = 32;          // largest cluster resolved as one block
 // A run of more than kClMax close values is cut into clusters, and pairs across a
-// cut keep angles of any size.  Applied together with everything else they
-// compose to anything but a rotation: the null space of a pencil of low rank or
-// of one with far more columns than rows (36 x 100: 64 zero values) took V to
-// 1e50 in four steps.  They are left alone instead (twice kBigAngle: the link
-// test is in FP32), so V stays orthogonal and every value outside the run
-// converges as ever; values within such a run stay as the Jacobi left them.
-constexpr double kMaxAngle = 2 * kBigAngle;
+// cut keep angles of any size.  A few such angles compose well enough for the
+// next steps to mend; where a column's add up to more than a limit they compose
+// to anything but a rotation: the null space of a pencil of low rank or of one
+// with far more columns than rows (36 x 100: 64 zero values, sums of 16 and
+// more) took V to 1e50 in four steps.  Such a column's angles above kBigAngle are
+// left alone, so that V stays near orthogonal and everything outside the run
+// converges as ever.  The limits fall from step to step, as nothing is left to
+// mend the last one's; pencils that converge stay below them (256 columns
+// graded over seven decades: 2.1, 0.9, 0.1, 0).
+constexpr int kRefineSteps = 4;
+constexpr float kCutAngles[kRefineSteps] = {3.f, 2.f, 0.5f, 0.f};
 constexpr int kClWarps = 8;         // clusters resolved at once
 
 __device__ __forceinline__ double oa_coupling(const double* K, const double* T, int c, int i, int j,
@@ -2215,12 +2220,14 @@ __device__ __forceinline__ double oa_coupling(const double* K, const double* T, 
 
 // F1 = I + (I - T)/2 + W, W the exact pair angles outside the clusters
 // (cid: cluster ids, -1 none); within a cluster only the orthogonality part.
+// wild: columns whose large angles are left alone (k_cluster_rot).
 // W itself goes to Wout: the caller adds W^2 / 2, so that I + W + W^2 / 2
 // (exp(W) to second order) is orthogonal up to W^4 / 4 — with I + W alone
 // the rotations' own W^2 defect (up to c kBigAngle^2) would have to be
 // squared away by the following steps.
 __global__ void k_oa_update(int c, const double* __restrict__ K, const double* __restrict__ T,
-                            const int* __restrict__ cid, double* __restrict__ F1, double* __restrict__ Wout) {
+                            const int* __restrict__ cid, const int* __restrict__ wild, double* __restrict__ F1,
+                            double* __restrict__ Wout) {
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= c * c) return;
   const int i = e % c, j = e / c;
@@ -2233,10 +2240,35 @@ __global__ void k_oa_update(int c, const double* __restrict__ K, const double* _
     const double cij = oa_coupling(K, T, c, i, j, li, lj);
     const double big = fmax(fabs(li), fabs(lj));
     if (fabs(lj - li) > kSepGap * big || fabs(cij) > kCoupleNoise * big) wij = 0.5 * atan(2.0 * cij / (lj - li));
-    if (fabs(wij) > kMaxAngle) wij = 0.0;
+    if (fabs(wij) > kBigAngle && (wild[i] || wild[j])) wij = 0.0;
   }
   F1[e] = f + wij;
   Wout[e] = wij;
+}
+
+// The columns whose angles across the cuts of long runs add up to more than
+// `limit` (k_cluster_rot's rare path, out of line for its registers; every
+// thread of the block calls it).  sum [c]: scratch in shared memory.
+__device__ __noinline__ void cut_sums(int c, const double* __restrict__ K, const double* __restrict__ T,
+                                      const float* lamf, const int* cid, float tb, float limit, int* sum, int* wild) {
+  const int tid = threadIdx.x;
+  for (int i = tid; i < c; i += blockDim.x) sum[i] = 0;
+  __syncthreads();
+  for (int j = tid >> 5; j < c; j += (int)(blockDim.x >> 5)) {
+    const float lj = lamf[j];
+    for (int i = tid & 31; i < j; i += 32) {
+      const float li = lamf[i], g = lj - li;
+      const float cij = (float)K[i + (size_t)j * c] - 0.5f * (li + lj) * (float)T[i + (size_t)j * c];
+      if (fabsf(2.f * cij) > tb * fabsf(g) && fabsf(cij) > (float)kCoupleNoise * fmaxf(fabsf(li), fabsf(lj)) &&
+          (cid[i] < 0 || cid[i] != cid[j])) {
+        const int a = (int)(0.5f * fabsf(atanf(2.f * cij / g)) * 65536.f);
+        atomicAdd(&sum[i], a);
+        atomicAdd(&sum[j], a);
+      }
+    }
+  }
+  __syncthreads();
+  for (int i = tid; i < c; i += blockDim.x) wild[i] = (float)sum[i] > limit * 65536.f;
 }
 
 // Cluster detection and resolution (one CTA).  Sorted by lam, a pair
@@ -2247,12 +2279,14 @@ __global__ void k_oa_update(int c, const double* __restrict__ K, const double* _
 // the size of the cluster's spread and couplings, so FP32 two-sided Jacobi on
 // it gives the rotation Q to FP32 relative accuracy (the next FP64 step
 // squares the rest away).  Outputs: cid (cluster id per index, -1 none),
-// ord / st (members of cluster q: ord[st[q] .. st[q+1]-1]) and Qb (c x c,
-// only the cluster blocks are written).
+// ord / st (members of cluster q: ord[st[q] .. st[q+1]-1]), Qb (c x c, only the
+// cluster blocks are written) and wild (1: the index's angles across the cuts of
+// longer runs add up to more than cut_angles; in fixed point, so in any order).
 __global__ void __launch_bounds__(1024) k_cluster_rot(int c, const double* __restrict__ K,
                                                       const double* __restrict__ T,
                                                       double* __restrict__ Qb, int* __restrict__ cid,
-                                                      int* __restrict__ ord, int* __restrict__ st) {
+                                                      int* __restrict__ ord, int* __restrict__ st,
+                                                      int* __restrict__ wild, float cut_angles) {
   extern __shared__ double cl_smem[];
   double* Sw = cl_smem;                                        // [kClWarps][kClMax][kClMax + 1]
   double* lam = Sw + kClWarps * kClMax * (kClMax + 1);         // [c]
@@ -2263,7 +2297,7 @@ __global__ void __launch_bounds__(1024) k_cluster_rot(int c, const double* __res
   int* pos = order + c;                                        // [c]
   int* link = pos + c;                                         // [c + 1] difference array of links
   int* start = link + c + 1;                                   // [c + 1]
-  __shared__ int s_ncl;
+  __shared__ int s_ncl, s_cut;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   for (int i = tid; i < c; i += blockDim.x) {
     // a zero (dropped) column has T_ii = 0: lambda 0 keeps the ranks below a permutation
@@ -2313,13 +2347,14 @@ __global__ void __launch_bounds__(1024) k_cluster_rot(int c, const double* __res
   }
   __syncthreads();
   if (tid == 0) {
-    int n = 0, len = 1, run = link[0];
+    int n = 0, len = 1, run = link[0], cut = 0;
     start[0] = 0;
     for (int k = 1; k < c; ++k) {
       // positions k-1 and k are linked when a large pair spans them
       if (run > 0 && len < kClMax) {
         ++len;
       } else {
+        cut |= run > 0;
         start[++n] = k;
         len = 1;
       }
@@ -2327,6 +2362,7 @@ __global__ void __launch_bounds__(1024) k_cluster_rot(int c, const double* __res
     }
     start[++n] = c;
     s_ncl = n;
+    s_cut = cut;
   }
   __syncthreads();
   const int ncl = s_ncl;
@@ -2334,6 +2370,9 @@ __global__ void __launch_bounds__(1024) k_cluster_rot(int c, const double* __res
     for (int k = start[q]; k < start[q + 1]; ++k) cid[order[k]] = (start[q + 1] - start[q] > 1) ? q : -1;
   for (int k = tid; k < c; k += blockDim.x) ord[k] = order[k];
   for (int q = tid; q <= ncl; q += blockDim.x) st[q] = start[q];
+  if (s_cut) cut_sums(c, K, T, lamf, cid, tb, cut_angles, link, wild);
+  else
+    for (int i = tid; i < c; i += blockDim.x) wild[i] = 0;
   if (warp >= kClWarps) return;
   float* B = Bw + (size_t)warp * kClMax * (kClMax + 1);
   float* Q = Qw + (size_t)warp * kClMax * (kClMax + 1);
@@ -2471,13 +2510,13 @@ static rr_status jacobi_svd(cudaStream_t s, int r, int c, const double* C, Penci
   k_v32_to_64<<<g, 256, 0, s>>>(c, cpad, w.V32, w.V);
   const size_t csm = cluster_smem(c);
   RR_TRY(allow_dynamic_smem((const void*)k_cluster_rot, csm));
-  constexpr int kRefineSteps = 4;
   for (int it = 0; it < kRefineSteps; ++it) {
     gemm_small(s, 0, 0, r, c, c, 1.0, C, r, w.V, c, 0.0, w.Mp, r);          // N = C V
     gemm_small_sym(s, c, r, w.Mp, r, w.Mp, r, w.E2, c);                     // K = N^T N
     gemm_small_sym(s, c, c, w.V, c, w.V, c, w.T, c);                        // T = V^T V
-    k_cluster_rot<<<1, 1024, csm, s>>>(c, w.E2, w.T, w.F, w.cid, w.order, w.cst);  // Qb
-    k_oa_update<<<gc, 256, 0, s>>>(c, w.E2, w.T, w.cid, w.Vp, w.E);         // F1, W
+    k_cluster_rot<<<1, 1024, csm, s>>>(c, w.E2, w.T, w.F, w.cid, w.order, w.cst, w.wild,
+                                        kCutAngles[it]);  // Qb
+    k_oa_update<<<gc, 256, 0, s>>>(c, w.E2, w.T, w.cid, w.wild, w.Vp, w.E);         // F1, W
     gemm_mixed(s, 0, 0, c, c, c, 0.5, w.E, c, w.E, c, 1.0, w.Vp, c);        // F1 += W^2 / 2
     // V <- V (I + (I - T)/2 + W) Qb: orthogonalise, the small pair rotations,
     // then the clusters' rotations

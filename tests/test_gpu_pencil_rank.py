@@ -60,6 +60,12 @@ def test_graded_columns(rr, b, decades):
     _check(rr, B, int((s > 1e-4 * s[0]).sum()))
 
 
+@pytest.mark.parametrize("b,decades", [(96, 9), (130, 8), (200, 7), (240, 7), (256, 6)])
+def test_graded_columns_that_separate(rr, b, decades):
+    """Small groups and mild angles across their cuts: every value and vector as accurate as any."""
+    _check(rr, _randn(b, b, seed=b) * torch.logspace(0, -decades, b, dtype=torch.float64), b)
+
+
 @pytest.mark.parametrize("spread", [0.0, 1e-8, 1e-5])
 def test_sixty_close_values(rr, spread):
     """60 of 120 values within `spread`: finite, orthonormal to 1e-5, values within the Jacobi's
