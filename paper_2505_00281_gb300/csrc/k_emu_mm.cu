@@ -50,7 +50,6 @@
 // Every wait is bounded (2 s); on expiry the kernel records an error, drains
 // its copies and MMAs, frees its TMEM and returns.
 #include <algorithm>
-#include <climits>
 #include <type_traits>
 
 #include "rr_common.cuh"
@@ -897,21 +896,24 @@ __global__ void __launch_bounds__(256) k_emu_col_exp(int64_t n, const TS* __rest
 }
 
 // Exponents of the largest entry of every row of a column-major block (lane =
-// row, 16 columns a thread at a time, atomic maxima; e starts very negative).
-template <typename TS>
+// row, 16 columns a thread, atomic maxima; e starts very negative).  kMore: the
+// grid strides over more columns than it has blocks for.
+template <typename TS, bool kMore>
 __global__ void __launch_bounds__(256) k_emu_row_exp(int64_t m, int64_t n, const TS* __restrict__ A, int64_t lda,
                                                      int* __restrict__ e) {
   const int64_t i = (int64_t)blockIdx.x * 32 + (threadIdx.x & 31);
-  if (i >= m) return;
-  int mx = INT_MIN;
-  for (int64_t j0 = ((int64_t)blockIdx.y * 8 + (threadIdx.x >> 5)) * 16; j0 < n; j0 += (int64_t)gridDim.y * 128) {
+  int64_t j0 = ((int64_t)blockIdx.y * 8 + (threadIdx.x >> 5)) * 16;
+  if (i >= m || j0 >= n) return;
+  do {
     typename Raw<TS>::R v[16];
 #pragma unroll
     for (int u = 0; u < 16; ++u) v[u] = j0 + u < n ? Raw<TS>::ld(A + i + (j0 + u) * lda) : 0;
+    int mx = kExpNone;
 #pragma unroll
     for (int u = 0; u < 16; ++u) mx = max(mx, exp_raw<TS>(v[u]));
-  }
-  if (mx > INT_MIN) atomicMax(e + i, mx);
+    atomicMax(e + i, mx);
+    j0 += (int64_t)gridDim.y * 128;
+  } while (kMore && j0 < n);
 }
 
 // G (p x q) = the sum of the K ranges' partial tiles in a fixed order (+ G).
@@ -1072,13 +1074,18 @@ rr_status col_exps(cudaStream_t s, int32_t type, int64_t n, int64_t c, const voi
 }
 
 rr_status row_exps(cudaStream_t s, int32_t type, int64_t n, int64_t c, const void* X, int64_t ldx, int* e) {
-  // (65535: the most blocks on y; the kernel strides over the columns beyond)
-  const dim3 g((unsigned)((n + 31) / 32), (unsigned)std::min<int64_t>((c + 127) / 128, 65535));
+  constexpr int64_t kMaxY = 65535;  // the most blocks on y
+  const dim3 g((unsigned)((n + 31) / 32), (unsigned)std::min<int64_t>((c + 127) / 128, kMaxY));
+  auto go = [&](auto ts) {
+    using TS = decltype(ts);
+    if (c > kMaxY * 128) k_emu_row_exp<TS, true><<<g, 256, 0, s>>>(n, c, (const TS*)X, ldx, e);
+    else k_emu_row_exp<TS, false><<<g, 256, 0, s>>>(n, c, (const TS*)X, ldx, e);
+  };
   switch (type) {
-    case RR_F64: k_emu_row_exp<double><<<g, 256, 0, s>>>(n, c, (const double*)X, ldx, e); break;
-    case RR_F32: k_emu_row_exp<float><<<g, 256, 0, s>>>(n, c, (const float*)X, ldx, e); break;
-    case RR_BF16: k_emu_row_exp<__nv_bfloat16><<<g, 256, 0, s>>>(n, c, (const __nv_bfloat16*)X, ldx, e); break;
-    case RR_E4M3: k_emu_row_exp<e4m3b_t><<<g, 256, 0, s>>>(n, c, (const e4m3b_t*)X, ldx, e); break;
+    case RR_F64: go(double{}); break;
+    case RR_F32: go(float{}); break;
+    case RR_BF16: go(__nv_bfloat16{}); break;
+    case RR_E4M3: go(e4m3b_t{}); break;
     default: return RR_ERR_ARG;
   }
   return check_launch("emu row exponents");
