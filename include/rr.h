@@ -362,8 +362,9 @@ rr_status rr_gemm_f64_emulated(int32_t trans, int64_t M, int64_t N, int64_t K, c
  * Needs rr_hessenberg_workspace_size(n, k, arith) bytes of workspace.
  * FP32: one launch where the block fits the CTAs' shared memory (one cluster
  * up to 16 CTAs, a cooperative grid above, panels of 8 columns, one exchange
- * per column), panels of 32 columns otherwise; FP64: one cooperative launch
- * with one grid barrier per column. */
+ * per column), panels of 32 columns otherwise (16 past 8.7 million rows on 152
+ * SMs, where no column is resident); FP64: one cooperative launch, the CTAs'
+ * candidates of a column gathered without a grid barrier. */
 size_t rr_hessenberg_workspace_size(int64_t n, int64_t k, int32_t arith);
 rr_status rr_hessenberg(int32_t arith, int64_t n, int64_t k, void* W, int64_t ldw,
                         int32_t qtype, void* Q, int64_t ldq, int32_t* piv, double tol,
@@ -379,8 +380,9 @@ rr_status rr_hessenberg(int32_t arith, int64_t n, int64_t k, void* W, int64_t ld
  * T -= L_panel W.  Every entry sees the same separately rounded operations in
  * the same order as in rr_hessenberg, so W, Q and piv equal its results bit
  * for bit; the trailing columns are streamed once per panel instead of once
- * per column.  rr_hessenberg takes this path by itself (panel 32) when a
- * CTA's share of rows of all k columns does not fit its shared memory.
+ * per column.  rr_hessenberg takes this path by itself (panel 32 or 16, see
+ * there) when a CTA's share of rows of all k columns does not fit its shared
+ * memory.
  * W: n x k FP32 (ld ldw, overwritten); Q: qtype RR_F32, RR_BF16 or RR_F64;
  * n < 2^24.  Workspace: rr_hessenberg_workspace_size(n, k, RR_F32).
  * RR_ERR_ARG: bad sizes, panel out of range, null pointers. */

@@ -304,27 +304,11 @@ __global__ void __launch_bounds__(kHessThreads) k_hessenberg(
   }
 }
 
-// the block's argmax from the per-warp candidates (the same merge order as
-// the warp-shuffle reduction, so every warp gets the same row)
-template <typename T>
-__device__ __forceinline__ int bi_of_block(const T* red_v, const int* red_i, int nwarps) {
-  T bv = T(-1);
-  int bi = INT_MAX;
-  const int lane = threadIdx.x & 31;
-  bv = lane < nwarps ? red_v[lane] : T(-1);
-  bi = lane < nwarps ? red_i[lane] : INT_MAX;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    T ov = __shfl_xor_sync(0xffffffffu, bv, o);
-    int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-    argmax_merge(bv, bi, ov, oi);
-  }
-  return bi;
-}
-
-// FP32-arithmetic variant (the basis step of the low-precision path), same
-// per-element arithmetic and results as k_hessenberg<float, TO>.  Two
-// changes to the per-column exchange:
+// FP32-arithmetic variant, same per-element arithmetic and results as
+// k_hessenberg<float, TO>: a block on one CTA (the batched solver's concurrent
+// problems), in shared memory where it fits, and the panels of blocks too tall
+// for one resident column, in memory on the whole grid; other FP32 blocks take
+// the resident kernels below.  Two changes to the per-column exchange:
 //   - a CTA's candidate is one 64-bit word (value bits, global row, column
 //     tag), written with a single release store and double-buffered by column
 //     parity, so the wait for the candidates also delivers them;

@@ -840,8 +840,9 @@ __global__ void k_whiten_corr(int b, double* __restrict__ E, const double* __res
 // this alone took rr_pencil_svd at 256 x 256 from 5.25 to 4.26 ms, at 320 x 320 (a
 // barrier over the grid instead of the cluster's) from 9.1 to 8.1 ms.
 // The rounding of the Gram entries is relative to the two columns' norms, far
-// below the 1e-4 the Jacobi stops at, and the next round starts from fresh
-// ones.  A pair whose inner product is exactly zero, or below tol relative to
+// below the 1e-4 the Jacobi stops at.  Cross products are formed anew in every
+// round; a block's own Gram matrix, norms included, is formed in a sweep's first
+// round and in the cluster form carried along from there.  A pair whose inner product is exactly zero, or below tol relative to
 // the column norms (floored, so rounding-level columns count as converged
 // against everything), is not rotated; zero columns (dropped directions,
 // padding) stay decoupled.  A round none of whose pairs would rotate skips its
