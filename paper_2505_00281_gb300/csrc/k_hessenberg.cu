@@ -1863,7 +1863,7 @@ template <typename TO>
 static rr_status hess_f32(int64_t n, int64_t k, float* W, int64_t ldw, TO* Q, int64_t ldq, int* piv, double tol,
                           void* ws, size_t ws_bytes, cudaStream_t s, int max_grid) {
   const HessPlan p = hess_plan(n, k);
-  if (max_grid == 1 || n == 0 || n >= (int64_t)kNoRow || (p.kr < 1 && k <= 16))
+  if (max_grid == 1 || n >= (int64_t)kNoRow || (p.kr < 1 && k <= 16))
     return hess_launch<float, TO>(n, k, W, ldw, Q, ldq, piv, tol, ws, ws_bytes, s, max_grid);
   if (p.kr < k) return hess_blocked<TO>(n, k, W, ldw, Q, ldq, piv, tol, p.kr < 1 ? 16 : kPanelMax, ws, ws_bytes, s);
   const size_t base = hess_ws_bytes<float>(k, num_sms());
@@ -1888,6 +1888,15 @@ namespace rr {
 rr_status hessenberg_ex(int32_t arith, int64_t n, int64_t k, void* W, int64_t ldw, int32_t qtype,
                         void* Q, int64_t ldq, int32_t* piv, double tol, void* ws, size_t ws_bytes,
                         cudaStream_t s, int max_grid);
+
+// A block without rows: every column is skipped (and no plan is made: it would
+// divide by the rows of a CTA).
+static rr_status hess_no_rows(int64_t k, int32_t* piv, void* ws, size_t ws_bytes, cudaStream_t s) {
+  if (!ws || ws_bytes < sizeof(int)) return RR_ERR_WORKSPACE;
+  RR_CUDA(cudaMemsetAsync(ws, 0, sizeof(int), s));  // the error word
+  RR_CUDA(cudaMemsetAsync(piv, 0xff, (size_t)k * sizeof(int32_t), s));
+  return RR_OK;
+}
 }
 extern "C" rr_status rr_hessenberg(int32_t arith, int64_t n, int64_t k, void* W, int64_t ldw,
                                    int32_t qtype, void* Q, int64_t ldq, int32_t* piv, double tol,
@@ -1902,6 +1911,9 @@ rr_status rr::hessenberg_ex(int32_t arith, int64_t n, int64_t k, void* W, int64_
   if (n < 0 || k < 0 || k > 4096 || ldw < n || ldq < n || !W || !Q || !piv) return RR_ERR_ARG;
   if (n > INT_MAX) return RR_ERR_ARG;
   if (k == 0) return RR_OK;
+  auto known = [](int32_t t, bool f8) { return t == RR_F64 || t == RR_F32 || t == RR_BF16 || (f8 && t == RR_E4M3); };
+  if (n == 0 && (arith == RR_F32 || arith == RR_F64) && known(qtype, arith == RR_F32))
+    return hess_no_rows(k, piv, ws, ws_bytes, s);
   if (arith == RR_F32) {
     float* w = (float*)W;
     switch (qtype) {
@@ -1928,6 +1940,7 @@ extern "C" rr_status rr_hessenberg_blocked(int64_t n, int64_t k, float* W, int64
   if (n >= (int64_t)kNoRow || panel < 1 || panel > kPanelMax) return RR_ERR_ARG;
   if (k == 0) return RR_OK;
   cudaStream_t s = as_stream(stream);
+  if (n == 0 && (qtype == RR_F32 || qtype == RR_BF16 || qtype == RR_F64)) return hess_no_rows(k, piv, ws, ws_bytes, s);
   switch (qtype) {
     case RR_F32: return hess_blocked<float>(n, k, W, ldw, (float*)Q, ldq, piv, tol, panel, ws, ws_bytes, s);
     case RR_BF16: return hess_blocked<__nv_bfloat16>(n, k, W, ldw, (__nv_bfloat16*)Q, ldq, piv, tol, panel, ws, ws_bytes, s);
