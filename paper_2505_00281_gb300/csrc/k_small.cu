@@ -1515,7 +1515,7 @@ struct PencilWs {
   double* cond;                        // [4] condition estimates of the whitened Grams, drop counts
   float *L32, *Li32, *M32, *V32, *fs;  // fs: [0] Jacobi norm floor, [1] scale
   float *Hq, *tq;                      // QR preconditioner: reflectors (c x c), taus
-  int *drop1, *drop2, *order, *nvalid, *rot, *err, *sweeps, *cid, *cst, *wild;
+  int *drop1, *drop2, *order, *nvalid, *rot, *err, *sweeps, *cid, *cst;
   GridBarrier* bar;
 };
 
@@ -1583,7 +1583,6 @@ static bool carve_pencil(Arena& ar, int b1, int b2, PencilWs& w) {
   w.sweeps = ar.take<int>(2);
   w.cid = ar.take<int>(cp);
   w.cst = ar.take<int>(cp + 1);
-  w.wild = ar.take<int>(cp);
   w.bar = ar.take<GridBarrier>(1);
   return !ar.overflow;
 }
@@ -2219,15 +2218,33 @@ __device__ __forceinline__ double oa_coupling(const double* K, const double* T, 
   return K[i + (size_t)j * c] - 0.5 * (li + lj) * T[i + (size_t)j * c];
 }
 
+// The large angles of column i across the cuts of long runs, added up (rare: only
+// elements with such an angle ask).  Columns i and j of a pair get the same sums
+// from either side of the diagonal.
+__device__ __noinline__ float cut_angles(int c, const double* __restrict__ K, const double* __restrict__ T,
+                                         const int* __restrict__ cid, int i) {
+  const float li = (float)(K[i + (size_t)i * c] / T[i + (size_t)i * c]);
+  float sum = 0.f;
+  for (int k = 0; k < c; ++k) {
+    if (k == i || (cid[i] >= 0 && cid[i] == cid[k])) continue;
+    const float lk = (float)(K[k + (size_t)k * c] / T[k + (size_t)k * c]);
+    const float cik = (float)K[k + (size_t)i * c] - 0.5f * (li + lk) * (float)T[k + (size_t)i * c];
+    if (!(fabsf(cik) > (float)kCoupleNoise * fmaxf(fabsf(li), fabsf(lk)))) continue;
+    const float a = 0.5f * fabsf(atanf(2.f * cik / (lk - li)));
+    if (a > (float)kBigAngle) sum += a;
+  }
+  return sum;
+}
+
 // F1 = I + (I - T)/2 + W, W the exact pair angles outside the clusters
 // (cid: cluster ids, -1 none); within a cluster only the orthogonality part.
-// wild: columns whose large angles are left alone (k_cluster_rot).
+// limit: kCutAngles of this step.
 // W itself goes to Wout: the caller adds W^2 / 2, so that I + W + W^2 / 2
 // (exp(W) to second order) is orthogonal up to W^4 / 4 — with I + W alone
 // the rotations' own W^2 defect (up to c kBigAngle^2) would have to be
 // squared away by the following steps.
 __global__ void k_oa_update(int c, const double* __restrict__ K, const double* __restrict__ T,
-                            const int* __restrict__ cid, const int* __restrict__ wild, double* __restrict__ F1,
+                            const int* __restrict__ cid, float limit, double* __restrict__ F1,
                             double* __restrict__ Wout) {
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= c * c) return;
@@ -2241,35 +2258,12 @@ __global__ void k_oa_update(int c, const double* __restrict__ K, const double* _
     const double cij = oa_coupling(K, T, c, i, j, li, lj);
     const double big = fmax(fabs(li), fabs(lj));
     if (fabs(lj - li) > kSepGap * big || fabs(cij) > kCoupleNoise * big) wij = 0.5 * atan(2.0 * cij / (lj - li));
-    if (fabs(wij) > kBigAngle && (wild[i] || wild[j])) wij = 0.0;
+    if (fabs(wij) > kBigAngle &&
+        (cut_angles(c, K, T, cid, i) > limit || cut_angles(c, K, T, cid, j) > limit))
+      wij = 0.0;
   }
   F1[e] = f + wij;
   Wout[e] = wij;
-}
-
-// The columns whose angles across the cuts of long runs add up to more than
-// `limit` (k_cluster_rot's rare path, out of line for its registers; every
-// thread of the block calls it).  sum [c]: scratch in shared memory.
-__device__ __noinline__ void cut_sums(int c, const double* __restrict__ K, const double* __restrict__ T,
-                                      const float* lamf, const int* cid, float tb, float limit, int* sum, int* wild) {
-  const int tid = threadIdx.x;
-  for (int i = tid; i < c; i += blockDim.x) sum[i] = 0;
-  __syncthreads();
-  for (int j = tid >> 5; j < c; j += (int)(blockDim.x >> 5)) {
-    const float lj = lamf[j];
-    for (int i = tid & 31; i < j; i += 32) {
-      const float li = lamf[i], g = lj - li;
-      const float cij = (float)K[i + (size_t)j * c] - 0.5f * (li + lj) * (float)T[i + (size_t)j * c];
-      if (fabsf(2.f * cij) > tb * fabsf(g) && fabsf(cij) > (float)kCoupleNoise * fmaxf(fabsf(li), fabsf(lj)) &&
-          (cid[i] < 0 || cid[i] != cid[j])) {
-        const int a = (int)(0.5f * fabsf(atanf(2.f * cij / g)) * 65536.f);
-        atomicAdd(&sum[i], a);
-        atomicAdd(&sum[j], a);
-      }
-    }
-  }
-  __syncthreads();
-  for (int i = tid; i < c; i += blockDim.x) wild[i] = (float)sum[i] > limit * 65536.f;
 }
 
 // Cluster detection and resolution (one CTA).  Sorted by lam, a pair
@@ -2280,14 +2274,12 @@ __device__ __noinline__ void cut_sums(int c, const double* __restrict__ K, const
 // the size of the cluster's spread and couplings, so FP32 two-sided Jacobi on
 // it gives the rotation Q to FP32 relative accuracy (the next FP64 step
 // squares the rest away).  Outputs: cid (cluster id per index, -1 none),
-// ord / st (members of cluster q: ord[st[q] .. st[q+1]-1]), Qb (c x c, only the
-// cluster blocks are written) and wild (1: the index's angles across the cuts of
-// longer runs add up to more than cut_angles; in fixed point, so in any order).
+// ord / st (members of cluster q: ord[st[q] .. st[q+1]-1]) and Qb (c x c,
+// only the cluster blocks are written).
 __global__ void __launch_bounds__(1024) k_cluster_rot(int c, const double* __restrict__ K,
                                                       const double* __restrict__ T,
                                                       double* __restrict__ Qb, int* __restrict__ cid,
-                                                      int* __restrict__ ord, int* __restrict__ st,
-                                                      int* __restrict__ wild, float cut_angles) {
+                                                      int* __restrict__ ord, int* __restrict__ st) {
   extern __shared__ double cl_smem[];
   double* Sw = cl_smem;                                        // [kClWarps][kClMax][kClMax + 1]
   double* lam = Sw + kClWarps * kClMax * (kClMax + 1);         // [c]
@@ -2298,7 +2290,7 @@ __global__ void __launch_bounds__(1024) k_cluster_rot(int c, const double* __res
   int* pos = order + c;                                        // [c]
   int* link = pos + c;                                         // [c + 1] difference array of links
   int* start = link + c + 1;                                   // [c + 1]
-  __shared__ int s_ncl, s_cut;
+  __shared__ int s_ncl;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   for (int i = tid; i < c; i += blockDim.x) {
     // a zero (dropped) column has T_ii = 0: lambda 0 keeps the ranks below a permutation
@@ -2348,14 +2340,13 @@ __global__ void __launch_bounds__(1024) k_cluster_rot(int c, const double* __res
   }
   __syncthreads();
   if (tid == 0) {
-    int n = 0, len = 1, run = link[0], cut = 0;
+    int n = 0, len = 1, run = link[0];
     start[0] = 0;
     for (int k = 1; k < c; ++k) {
       // positions k-1 and k are linked when a large pair spans them
       if (run > 0 && len < kClMax) {
         ++len;
       } else {
-        cut |= run > 0;
         start[++n] = k;
         len = 1;
       }
@@ -2363,7 +2354,6 @@ __global__ void __launch_bounds__(1024) k_cluster_rot(int c, const double* __res
     }
     start[++n] = c;
     s_ncl = n;
-    s_cut = cut;
   }
   __syncthreads();
   const int ncl = s_ncl;
@@ -2371,9 +2361,6 @@ __global__ void __launch_bounds__(1024) k_cluster_rot(int c, const double* __res
     for (int k = start[q]; k < start[q + 1]; ++k) cid[order[k]] = (start[q + 1] - start[q] > 1) ? q : -1;
   for (int k = tid; k < c; k += blockDim.x) ord[k] = order[k];
   for (int q = tid; q <= ncl; q += blockDim.x) st[q] = start[q];
-  if (s_cut) cut_sums(c, K, T, lamf, cid, tb, cut_angles, link, wild);
-  else
-    for (int i = tid; i < c; i += blockDim.x) wild[i] = 0;
   if (warp >= kClWarps) return;
   float* B = Bw + (size_t)warp * kClMax * (kClMax + 1);
   float* Q = Qw + (size_t)warp * kClMax * (kClMax + 1);
@@ -2515,9 +2502,8 @@ static rr_status jacobi_svd(cudaStream_t s, int r, int c, const double* C, Penci
     gemm_small(s, 0, 0, r, c, c, 1.0, C, r, w.V, c, 0.0, w.Mp, r);          // N = C V
     gemm_small_sym(s, c, r, w.Mp, r, w.Mp, r, w.E2, c);                     // K = N^T N
     gemm_small_sym(s, c, c, w.V, c, w.V, c, w.T, c);                        // T = V^T V
-    k_cluster_rot<<<1, 1024, csm, s>>>(c, w.E2, w.T, w.F, w.cid, w.order, w.cst, w.wild,
-                                        kCutAngles[it]);  // Qb
-    k_oa_update<<<gc, 256, 0, s>>>(c, w.E2, w.T, w.cid, w.wild, w.Vp, w.E);         // F1, W
+    k_cluster_rot<<<1, 1024, csm, s>>>(c, w.E2, w.T, w.F, w.cid, w.order, w.cst);  // Qb
+    k_oa_update<<<gc, 256, 0, s>>>(c, w.E2, w.T, w.cid, kCutAngles[it], w.Vp, w.E);         // F1, W
     gemm_mixed(s, 0, 0, c, c, c, 0.5, w.E, c, w.E, c, 1.0, w.Vp, c);        // F1 += W^2 / 2
     // V <- V (I + (I - T)/2 + W) Qb: orthogonalise, the small pair rotations,
     // then the clusters' rotations
