@@ -194,9 +194,10 @@ def aggregate(seconds: float, converged: int, dist=None, device=None):
 # DRAM bytes per launch by role (the low-precision products of k_gemm_bf16_tc;
 # the FP64-emulation passes of k_emu_mm), mean over one solve of this workload (ncu
 # dram__bytes_read.sum + dram__bytes_write.sum, a one-pass capture of every
-# launch of the kernel in one solve; profiles/ncu_gemm_bf16_tc_16384x4096x128.md).
+# launch of the kernel in one solve; profiles/ncu_gemm_bf16_tc_16384x4096x128.md and
+# profiles/ncu_emu_mm_16384x4096x128.md).
 # Emptied when the kernel changes, until it is captured again.
-TC_TRAFFIC_PER_LAUNCH = {"lowp_product": 221.6e6}
+TC_TRAFFIC_PER_LAUNCH = {"lowp_product": 221.6e6, "f64_emulation": 120.8e6}
 
 
 def stage_roofline(info, peaks, src):
