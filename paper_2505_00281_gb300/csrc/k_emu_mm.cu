@@ -870,7 +870,7 @@ __global__ void __launch_bounds__(256) k_emu_bslice(int64_t K, int64_t N, const 
 template <typename TS>
 __global__ void __launch_bounds__(256) k_emu_col_exp(int64_t n, const TS* __restrict__ X, int64_t ldx, int64_t rpc,
                                                      int* __restrict__ e) {
-  const int64_t j = blockIdx.x, r0 = (int64_t)blockIdx.y * rpc, r1 = min(n, r0 + rpc);
+  const int64_t j = blockIdx.y, r0 = (int64_t)blockIdx.x * rpc, r1 = min(n, r0 + rpc);
   const TS* x = X + j * ldx;
   int mx = kExpNone;
   for (int64_t i = r0 + threadIdx.x; i < r1; i += 8 * 256) {
@@ -881,7 +881,7 @@ __global__ void __launch_bounds__(256) k_emu_col_exp(int64_t n, const TS* __rest
     for (int u = 0; u < 8; ++u) mx = max(mx, exp_raw<TS>(v[u]));
   }
   mx = __reduce_max_sync(0xffffffffu, mx);
-  if (gridDim.y > 1) {
+  if (gridDim.x > 1) {
     if ((threadIdx.x & 31) == 0) atomicMax(e + j, mx);
     return;
   }
@@ -1058,27 +1058,35 @@ int64_t col_exp_chunks(int64_t n, int64_t c) {
   if (n <= 4096) return 1;
   return std::max<int64_t>(1, std::min<int64_t>((n + 2047) / 2048, (8 * (int64_t)num_sms() + c - 1) / c));
 }
+constexpr int64_t kMaxGridY = 65535;
 rr_status col_exps(cudaStream_t s, int32_t type, int64_t n, int64_t c, const void* X, int64_t ldx, int* e) {
   int64_t chunks = col_exp_chunks(n, c);
   const int64_t rpc = (n + chunks - 1) / chunks;
   chunks = (n + rpc - 1) / rpc;
-  const dim3 g((unsigned)c, (unsigned)chunks);
-  switch (type) {
-    case RR_F64: k_emu_col_exp<double><<<g, 256, 0, s>>>(n, (const double*)X, ldx, rpc, e); break;
-    case RR_F32: k_emu_col_exp<float><<<g, 256, 0, s>>>(n, (const float*)X, ldx, rpc, e); break;
-    case RR_BF16: k_emu_col_exp<__nv_bfloat16><<<g, 256, 0, s>>>(n, (const __nv_bfloat16*)X, ldx, rpc, e); break;
-    case RR_E4M3: k_emu_col_exp<e4m3b_t><<<g, 256, 0, s>>>(n, (const e4m3b_t*)X, ldx, rpc, e); break;
-    default: return RR_ERR_ARG;
+  // columns on y, in as many launches as that takes (an operator may have millions)
+  for (int64_t j0 = 0; j0 < c; j0 += kMaxGridY) {
+    const dim3 g((unsigned)chunks, (unsigned)std::min<int64_t>(c - j0, kMaxGridY));
+    auto go = [&](auto ts) {
+      using TS = decltype(ts);
+      k_emu_col_exp<TS><<<g, 256, 0, s>>>(n, (const TS*)X + j0 * ldx, ldx, rpc, e + j0);
+    };
+    switch (type) {
+      case RR_F64: go(double{}); break;
+      case RR_F32: go(float{}); break;
+      case RR_BF16: go(__nv_bfloat16{}); break;
+      case RR_E4M3: go(e4m3b_t{}); break;
+      default: return RR_ERR_ARG;
+    }
+    RR_TRY(check_launch("emu column exponents"));
   }
-  return check_launch("emu column exponents");
+  return RR_OK;
 }
 
 rr_status row_exps(cudaStream_t s, int32_t type, int64_t n, int64_t c, const void* X, int64_t ldx, int* e) {
-  constexpr int64_t kMaxY = 65535;  // the most blocks on y
-  const dim3 g((unsigned)((n + 31) / 32), (unsigned)std::min<int64_t>((c + 127) / 128, kMaxY));
+  const dim3 g((unsigned)((n + 31) / 32), (unsigned)std::min<int64_t>((c + 127) / 128, kMaxGridY));
   auto go = [&](auto ts) {
     using TS = decltype(ts);
-    if (c > kMaxY * 128) k_emu_row_exp<TS, true><<<g, 256, 0, s>>>(n, c, (const TS*)X, ldx, e);
+    if (c > kMaxGridY * 128) k_emu_row_exp<TS, true><<<g, 256, 0, s>>>(n, c, (const TS*)X, ldx, e);
     else k_emu_row_exp<TS, false><<<g, 256, 0, s>>>(n, c, (const TS*)X, ldx, e);
   };
   switch (type) {
